@@ -106,9 +106,11 @@ struct ichee_ctx {
     int8_t* d_s = nullptr;
     int8_t* d_srev = nullptr;
     u64* d_pk = nullptr;         // [2][L][N]
-    u64* d_pk_hat = nullptr;
-    u64* d_pk_hat_p = nullptr;
-    ulonglong2* d_pk_pair = nullptr;   // (pk_hat, pk_hat_p) interleaved: the encryption kernel's operand
+    ichee::AuxPrimes aux = {};   // auxiliary primes of fresh encryption, tables inside d_aux_tables
+    uint2* d_aux_tables = nullptr;   // [aux.n][2][N]: forward then inverse twiddles
+    ichee::EncLimb enc_limb[kMaxPrimes] = {};
+    int enc_units = 0;
+    u32* d_pk_aux = nullptr;     // [enc_units][2][N]: the encryption kernel's key operands
     u64* d_evk = nullptr;        // [L][2][L+1][N]
     u64* d_evk_hat = nullptr;
     u64* d_evk_hat_p = nullptr;

@@ -38,6 +38,13 @@ __device__ __forceinline__ u64 shoup(u64 x, u64 w, u64 wp, u64 q)
 
 __device__ __forceinline__ u64 csub(u64 x, u64 q) { return x >= q ? x - q : x; }
 
+// The same for x, q < 2^63: the sign of the difference decides, one comparison of high words.
+__device__ __forceinline__ u64 csub_s(u64 x, u64 q)
+{
+    const i64 d = (i64)(x - q);
+    return d < 0 ? x : (u64)d;
+}
+
 __device__ __forceinline__ u64 add_mod(u64 a, u64 b, u64 q) { return csub(a + b, q); }
 
 __device__ __forceinline__ u64 sub_mod(u64 a, u64 b, u64 q) { return a >= b ? a - b : a + q - b; }
@@ -97,8 +104,8 @@ __device__ __forceinline__ Words4 philox(u64 seed, u32 stream, u64 id, u32 block
 #pragma unroll
     for (int round = 0; round < 10; ++round) {
         if (round > 0) { k0 += 0x9E3779B9u; k1 += 0xBB67AE85u; }
-        u32 hi0 = __umulhi(0xD2511F53u, c0), lo0 = 0xD2511F53u * c0;
-        u32 hi1 = __umulhi(0xCD9E8D57u, c2), lo1 = 0xCD9E8D57u * c2;
+        const u64 p0 = (u64)0xD2511F53u * c0, p1 = (u64)0xCD9E8D57u * c2;   // one wide multiply each
+        const u32 hi0 = (u32)(p0 >> 32), lo0 = (u32)p0, hi1 = (u32)(p1 >> 32), lo1 = (u32)p1;
         u32 n0 = hi1 ^ c1 ^ k0;
         u32 n2 = hi0 ^ c3 ^ k1;
         c0 = n0; c1 = lo1; c2 = n2; c3 = lo0;
@@ -114,8 +121,8 @@ enum Stream : u32 {
     kStreamKeyS = 8, kStreamKeyE = 9, kStreamKeyA = 16
 };
 
-// Uniform ternary from one 32-bit word: floor(3w / 2^32) - 1.
-__device__ __forceinline__ int ternary_of(u32 w) { return (int)(((u64)w * 3u) >> 32) - 1; }
+// Uniform ternary from one 32-bit word: floor(3w / 2^32) - 1, by the two words where it steps.
+__device__ __forceinline__ int ternary_of(u32 w) { return (w >= 0xAAAAAAABu ? 1 : 0) - (w < 0x55555556u ? 1 : 0); }
 
 // Discrete Gaussian from one 64-bit value: top bit sign, magnitude = number of table
 // entries the low 63 bits reach (table strictly increasing, last entry 2^63).

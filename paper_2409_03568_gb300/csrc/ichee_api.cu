@@ -135,6 +135,8 @@ void ichee::encode_const(const ichee_ctx* c, double value, double scale, int lim
 // ---------------------------------------------------------------------------------------
 // Context
 // ---------------------------------------------------------------------------------------
+static ichee_status make_aux(ichee_ctx* c);
+
 extern "C" ichee_status ichee_ctx_create(const ichee_params* p, int device, ichee_ctx** out)
 {
     if (!p || !out) return fail(ICHEE_EINVAL, "ichee_ctx_create: null argument");
@@ -276,6 +278,8 @@ extern "C" ichee_status ichee_ctx_create(const ichee_params* p, int device, iche
             cl.mu[i] = (u64)(((hm::u128)1 << 64) / c->q[i]);
         }
     }
+    const ichee_status aux_st = make_aux(c);
+    if (aux_st != ICHEE_OK) return cleanup(aux_st);
     if (cudaMalloc(&c->d_status, sizeof(int)) != cudaSuccess) return cleanup(fail(ICHEE_ENOMEM, "status"));
     cudaMemset(c->d_status, 0, sizeof(int));
     if (cudaGetLastError() != cudaSuccess) return cleanup(fail(ICHEE_ECUDA, "context set-up"));
@@ -288,7 +292,7 @@ extern "C" void ichee_ctx_destroy(ichee_ctx* c)
     if (!c) return;
     cudaSetDevice(c->device);
     cudaDeviceSynchronize();
-    void* ptrs[] = {c->d_tables, c->d_half_tw, c->d_dm, c->d_ninv, c->d_s, c->d_srev, c->d_pk, c->d_pk_hat, c->d_pk_hat_p, c->d_pk_pair,
+    void* ptrs[] = {c->d_tables, c->d_half_tw, c->d_dm, c->d_ninv, c->d_s, c->d_srev, c->d_pk, c->d_aux_tables, c->d_pk_aux,
                     c->d_evk, c->d_evk_hat, c->d_evk_hat_p, c->d_status};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -317,6 +321,95 @@ extern "C" ichee_status ichee_ct_bytes(const ichee_ctx* c, uint32_t level, size_
     return ICHEE_OK;
 }
 
+// Auxiliary primes, their tables and the per-limb constants of fresh encryption (ntt32.cuh).
+// A limb takes two primes while N q / 2 (the largest coefficient of v * pk) is at most M / 4, else
+// three, which suffice for every supported N and q; M / 4 leaves the rounding of k its margin.
+static ichee_status make_aux(ichee_ctx* c)
+{
+    std::vector<u64> taken;
+    for (int i = 0; i < kAuxMax; ++i) {
+        const u64 p = hm::chain_prime(kAuxBits, (unsigned)c->logn, taken);
+        if (!p || (1ull << kAuxBits) - p > (1ull << 22)) return fail(ICHEE_EUNSUPPORTED, "no auxiliary prime");
+        taken.push_back(p);
+        c->aux.p[i] = (u32)p;
+        u32 inv = (u32)p;                   // Newton iteration for p^{-1} mod 2^32 (p odd)
+        for (int it = 0; it < 5; ++it) inv *= 2u - (u32)p * inv;
+        c->aux.pinv[i] = inv;
+    }
+    c->aux.n = 2;
+    c->enc_units = 0;
+    for (int l = 0; l < c->L; ++l) {
+        EncLimb& e = c->enc_limb[l];
+        const u64 q = c->q[l];
+        e.q = q;
+        const hm::u128 m2 = (hm::u128)taken[0] * taken[1];
+        e.np = (hm::u128)c->n * (q / 2) <= m2 / 4 ? 2 : 3;
+        e.unit = c->enc_units;
+        c->enc_units += e.np;
+        c->aux.n = std::max(c->aux.n, e.np);
+        e.bits = (int)c->params.prime_bits[l];
+        e.t = e.bits > 32 ? e.bits - 1 - 32 : e.bits - 1;
+        e.mu = (u32)(((hm::u128)1 << (e.bits + 31)) / q);
+        e.p_last = c->aux.p[e.np - 1];
+        e.nq_lo = (u32)(0 - q);
+        e.nq_hi = (u32)((0 - q) >> 32);
+        u64 m_last = 1;
+        for (int i = 0; i < e.np; ++i) {    // M / p_i mod q
+            u64 mi = 1;
+            for (int j = 0; j < e.np; ++j)
+                if (j != i) mi = hm::mulm(mi, taken[j] % q, q);
+            e.ml[i] = (u32)mi;
+            e.mh[i] = (u32)(mi >> 32);
+            m_last = mi;
+        }
+        e.c0 = 2 * q - 32 - hm::mulm(5ull * e.p_last % q, m_last, q);
+    }
+    const size_t n = (size_t)c->n;
+    if (cudaMalloc(&c->d_aux_tables, (size_t)c->aux.n * 2 * n * sizeof(uint2)) != cudaSuccess)
+        return fail(ICHEE_ENOMEM, "auxiliary tables");
+    std::vector<uint2> t(2 * n);
+    for (int i = 0; i < c->aux.n; ++i) {
+        const u64 p = taken[i], psi = hm::root_2n(p, (unsigned)c->logn), psi_inv = hm::invm(psi, p);
+        u64 w = 1, iw = 1;
+        for (size_t k = 0; k < n; ++k) {
+            const unsigned r = hm::bitrev((unsigned)k, (unsigned)c->logn);
+            t[r] = make_uint2((u32)w, (u32)((w << 32) / p));
+            t[n + r] = make_uint2((u32)iw, (u32)((iw << 32) / p));
+            w = w * psi % p;
+            iw = iw * psi_inv % p;
+        }
+        uint2* d = c->d_aux_tables + (size_t)i * 2 * n;
+        if (cudaMemcpy(d, t.data(), 2 * n * sizeof(uint2), cudaMemcpyHostToDevice) != cudaSuccess)
+            return fail(ICHEE_ECUDA, "upload auxiliary tables");
+        c->aux.tw[i] = d;
+        c->aux.itw[i] = d + n;
+    }
+    return ICHEE_OK;
+}
+
+static PkAuxArgs pk_aux_args(const ichee_ctx* c)
+{
+    PkAuxArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.aux = c->aux;
+    a.L = c->L;
+    a.pk = c->d_pk;
+    a.out = c->d_pk_aux;
+    for (int l = 0; l < c->L; ++l) {
+        const EncLimb& e = c->enc_limb[l];
+        a.unit[l] = e.unit;
+        a.q[l] = e.q;
+        for (int i = 0; i < e.np; ++i) {
+            const u64 p = c->aux.p[i];
+            u64 m = (u64)c->n % p;          // N M / p_i mod p_i
+            for (int j = 0; j < e.np; ++j)
+                if (j != i) m = m * c->aux.p[j] % p;
+            a.k[e.unit + i] = (u32)(hm::invm(m, p) * ((1ull << 32) % p) % p);
+        }
+    }
+    return a;
+}
+
 // ---------------------------------------------------------------------------------------
 // Key generation (Sec. 2.2.2: pk = (-a*s + e, a); evk for hybrid key switching with the
 // special prime P, one digit per ciphertext prime)
@@ -330,9 +423,7 @@ static cudaError_t alloc_key_buffers(ichee_ctx* c)
         if ((e = cudaMalloc(&c->d_s, c->n)) != cudaSuccess) return e;
         if ((e = cudaMalloc(&c->d_srev, c->n)) != cudaSuccess) return e;
         if ((e = cudaMalloc(&c->d_pk, 2 * c->L * polyb)) != cudaSuccess) return e;
-        if ((e = cudaMalloc(&c->d_pk_hat, 2 * c->L * polyb)) != cudaSuccess) return e;
-        if ((e = cudaMalloc(&c->d_pk_hat_p, 2 * c->L * polyb)) != cudaSuccess) return e;
-        if ((e = cudaMalloc(&c->d_pk_pair, 4 * c->L * polyb)) != cudaSuccess) return e;
+        if ((e = cudaMalloc(&c->d_pk_aux, (size_t)c->enc_units * polyb)) != cudaSuccess) return e;
     }
     return e;
 }
@@ -385,12 +476,7 @@ extern "C" ichee_status ichee_keygen(ichee_ctx* c, uint64_t seed, uint32_t flags
     KCK(launch_ntt_inv(rl, batch(A, L, L, id.data()), st));
     KCK(launch_scale_const(rl, batch(A, L, L, id.data()), c->d_ninv, st));
     for (int l = 0; l < L; ++l) KCK(launch_neg_add_small(A + (size_t)l * n, d_e, n, c->q[l], pk0 + (size_t)l * n, st));
-    // pk^ = NTT(pk) * N^{-1} with Shoup companions (the encryption kernel's operands)
-    KCK(cudaMemcpyAsync(c->d_pk_hat, c->d_pk, 2 * L * polyb, cudaMemcpyDeviceToDevice, st));
-    KCK(launch_ntt_fwd(rl, batch(c->d_pk_hat, 2 * L, L, id.data()), st));
-    KCK(launch_scale_const(rl, batch(c->d_pk_hat, 2 * L, L, id.data()), c->d_ninv, st));
-    KCK(launch_shoup_companions(rl, batch(c->d_pk_hat, 2 * L, L, id.data()), c->d_pk_hat_p, st));
-    KCK(launch_interleave(c->d_pk_hat, c->d_pk_hat_p, (u64)2 * L * c->n, c->d_pk_pair, st));
+    KCK(launch_pk_aux(pk_aux_args(c), c->logn, c->enc_units, st));
 
     // s on the host: export copy and the reversed-negated form used by decryption
     c->h_s.resize(n);
@@ -509,13 +595,8 @@ extern "C" ichee_status ichee_import_key(ichee_ctx* c, int which, const void* ho
             for (int l = 0; l < L; ++l)
                 for (int j = 0; j < n; ++j)
                     if (k[((size_t)b * L + l) * n + j] >= c->q[l]) return fail(ICHEE_EINVAL, "public key residue out of range");
-        const RnsArgs rl = rns_prefix(c, L);
         CK(cudaMemcpyAsync(c->d_pk, k, 2 * L * polyb, cudaMemcpyHostToDevice, st));
-        CK(cudaMemcpyAsync(c->d_pk_hat, c->d_pk, 2 * L * polyb, cudaMemcpyDeviceToDevice, st));
-        CK(launch_ntt_fwd(rl, batch(c->d_pk_hat, 2 * L, L, id.data()), st));
-        CK(launch_scale_const(rl, batch(c->d_pk_hat, 2 * L, L, id.data()), c->d_ninv, st));
-        CK(launch_shoup_companions(rl, batch(c->d_pk_hat, 2 * L, L, id.data()), c->d_pk_hat_p, st));
-        CK(launch_interleave(c->d_pk_hat, c->d_pk_hat_p, (u64)2 * L * c->n, c->d_pk_pair, st));
+        CK(launch_pk_aux(pk_aux_args(c), c->logn, c->enc_units, st));
         CK(cudaStreamSynchronize(st));
         c->have_pk = true;
         return ICHEE_OK;
@@ -556,12 +637,14 @@ EncArgs ichee::enc_args(const ichee_ctx* c, const uint8_t* d_pix, u64 n_ct, u64 
 {
     EncArgs a;
     std::memset(&a, 0, sizeof(a));
-    a.rns = rns_prefix(c, c->L);
+    a.logn = c->logn;
     a.L = c->L;
+    a.aux = c->aux;
+    for (int l = 0; l < c->L; ++l) a.limb[l] = c->enc_limb[l];
     a.n_ct = n_ct;
     a.pixels = d_pix;
     a.dm = c->d_dm;
-    a.pk_pair = c->d_pk_pair;
+    a.pk_aux = c->d_pk_aux;
     a.skip_lut = nullptr;
     a.seed = seed;
     a.id_base = id_base;

@@ -8,30 +8,65 @@ namespace ichee {
 constexpr int kMinLogN = 10;
 constexpr int kMaxLogN = 14;
 
+// Auxiliary primes of the fresh-encryption products (ntt32.cuh): primes just below 2^28, = 1 mod
+// 2N, with their transform tables (twiddle, Shoup companion floor(w 2^32 / p)).
+constexpr int kAuxBits = 28;
+constexpr int kAuxMax = 3;
+struct AuxPrimes {
+    int n;                          // primes in use (2 or 3)
+    u32 p[kAuxMax], pinv[kAuxMax];  // p^{-1} mod 2^32
+    const uint2* tw[kAuxMax];       // [N] psi^{bitrev(k)}
+    const uint2* itw[kAuxMax];      // [N] psi^{-bitrev(k)}
+};
+
+// Constants of one ciphertext limb for the exact product (enc_crt): np auxiliary primes with
+// product M, unit the index of the limb's first (limb, prime) pair; ml / mh the low and high words
+// of M / p_i mod q, p_last = p_{np-1}, c0 = 2q - 32 - (5 p_last M / p_last mod q),
+// mu = floor(2^(bits + 31) / q), nq_lo / nq_hi the words of 2^64 - q, and T = V >> (bits - 1) is taken
+// as (V >> 32) >> t (a limb of at most 32 bits: V >> t).
+struct EncLimb {
+    u64 q, c0;
+    int np, unit, bits, t;
+    u32 ml[kAuxMax], mh[kAuxMax], mu, p_last, nq_lo, nq_hi;
+};
+
 // Fresh public-key encryption of pixel values (Sec. 2.2.2, 3.1).
 struct EncArgs {
-    RnsArgs rns;               // moduli 0..L-1 = ciphertext primes
+    int logn;
     int L;                     // limbs written
+    AuxPrimes aux;
+    EncLimb limb[kMaxPrimes];
     u64 n_ct;                  // ciphertexts
     const uint8_t* pixels;     // [n_ct] device
     const u64* dm;             // [L][256] (Delta * p) mod q_l
-    const ulonglong2* pk_pair; // [2][L][N] (NTT(pk_b) * N^{-1}, its Shoup companion), bit-reversed order
+    const u32* pk_aux;         // the key modulo the auxiliary primes, transformed (launch_pk_aux)
     const int32_t* skip_lut;   // optional [256]: skip pixel p when skip_lut[p] >= 0
     u64 seed;
     u64 id_base;               // ct id of ciphertext k is id_base + k
     CdtTable cdt;
     u64* out;                  // [n_ct][2][L][N]
-    int num_sms;               // persistent grid of the single-image kernel: one block per SM
+    int num_sms;               // persistent grid of the single-image kernel
     const u32* idx;            // optional: encrypt only pixels idx[0 .. *n_idx) (device list)
     const u32* n_idx;
 };
 
+// Key operands of fresh encryption from the public key [2][L][N] (see k_pk_aux): n_units x 2 x N
+// words; k[u] = N^{-1} (M / p_i)^{-1} 2^32 mod p_i for unit u.
+constexpr int kMaxEncUnits = 3 * kMaxPrimes;
+struct PkAuxArgs {
+    AuxPrimes aux;
+    int L;
+    int unit[kMaxPrimes];
+    u64 q[kMaxPrimes];
+    u32 k[kMaxEncUnits];
+    const u64* pk;
+    u32* out;
+};
+cudaError_t launch_pk_aux(const PkAuxArgs& a, int logn, int n_units, cudaStream_t st);
+
 // idx[0 .. *count) = the pixels k < n whose value has no slot (lut[px[k]] < 0), in any order;
 // *count is zeroed first. Everything on the stream.
 cudaError_t launch_miss_list(const uint8_t* px, u64 n, const int32_t* lut, u32* idx, u32* count, cudaStream_t st);
-
-// pair[i] = (a[i], b[i]) for i < n
-cudaError_t launch_interleave(const u64* a, const u64* b, u64 n, ulonglong2* pair, cudaStream_t st);
 
 // Radix-cached encryption: c = sum_k M[k][d'_k], M[k][d] = d * Enc(r^k) (Sec. 3.2, 3.3).
 struct RadixArgs {

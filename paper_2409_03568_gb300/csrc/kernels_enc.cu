@@ -1,9 +1,36 @@
 // kernels_enc.cu -- key generation helpers, fused fresh encryption (Sec. 2.2.2, 3.1) and the
 // cached encryption kernels (radix combine and value lookup with the zero pool, Sec. 3.2, 3.3).
 #include "internal.h"
-#include "ntt.cuh"
+#include "ntt32.cuh"
 
 namespace ichee {
+
+// Shape of the fresh-encryption kernel. Up to N = 2^13: 8 residues per thread, both polynomials
+// of a limb in lockstep (each twiddle loaded once for the two, exchanges in 64-bit words); at
+// N = 2^14 (1024 threads, 16 residues) one polynomial at a time, as two take more than the 64
+// registers. Blocks of up to 1024 threads in 64 registers a thread, as many per SM as that allows.
+// 16 residues in 128 registers were slower at N = 2^13 (102 against 96 us per ciphertext and SM) and
+// at 2^12 (61 against 51), as was a second set of samples drawn ahead (96.4 against 95.9).
+template <int LOGN>
+struct EncShape {
+    static constexpr int N = 1 << LOGN;
+    static constexpr int E = LOGN <= 13 ? 8 : 16;
+    static constexpr int T = N / E;
+    static constexpr int NP = LOGN <= 13 ? 2 : 1;
+    static constexpr int KEEP = 2;   // v^ modulo two primes at a time
+    static constexpr int BLOCKS = 1024 / T;
+    static constexpr size_t CDT_AT = (size_t)N * (4 * NP + 4 * KEEP + 2);
+    static constexpr size_t SMEM = CDT_AT + 32 * sizeof(u64);
+    static_assert(SMEM <= 227 * 1024 && BLOCKS * (SMEM + 1024) <= 228 * 1024, "shared memory of an SM");
+};
+
+// Word of the key operands for unit u, polynomial b, transform position x: both polynomials of a
+// position adjacent where they are transformed together.
+template <int LOGN>
+__host__ __device__ constexpr size_t enc_pk_at(int u, int b, int x)
+{
+    return EncShape<LOGN>::NP == 2 ? (((size_t)u << LOGN) + x) * 2 + b : (((size_t)u * 2 + b) << LOGN) + x;
+}
 
 // ---------------------------------------------------------------------------------------
 // Samplers (Sec. 2.2.1 / 2.2.2). Coefficient i of a ternary polynomial uses word i%4 of
@@ -217,19 +244,6 @@ __global__ void k_axpy_const(u64* out, const u64* x, const u64* y, u64 c, int n,
     if (i < n) out[i] = add_mod(x[i], mul_mod(c, y[i], q, m0, m1), q);
 }
 
-__global__ void k_interleave(const u64* a, const u64* b, u64 n, ulonglong2* pair)
-{
-    for (u64 i = blockIdx.x * (u64)blockDim.x + threadIdx.x; i < n; i += (u64)gridDim.x * blockDim.x)
-        pair[i] = make_ulonglong2(a[i], b[i]);
-}
-
-cudaError_t launch_interleave(const u64* a, const u64* b, u64 n, ulonglong2* pair, cudaStream_t st)
-{
-    const u64 blocks = (n + 255) / 256;
-    k_interleave<<<(unsigned)(blocks < 4096 ? blocks : 4096), 256, 0, st>>>(a, b, n, pair);
-    return cudaGetLastError();
-}
-
 cudaError_t launch_axpy_const(u64* out, const u64* x, const u64* y, u64 c, int n, u64 q, u64 m0, u64 m1,
                               cudaStream_t st)
 {
@@ -238,167 +252,241 @@ cudaError_t launch_axpy_const(u64* out, const u64* x, const u64* y, u64 c, int n
 }
 
 // ---------------------------------------------------------------------------------------
-// Fused fresh encryption (Sec. 2.2.2, with the library sign convention pk = (-a*s + e, a),
-// since the printed formulas do not cancel): one thread block per ciphertext.
-//   sample v (ternary), e0, e1 (Gaussian) once into shared memory (int8), then per limb l:
-//   v^ = NTT(v); c_b = INTT(v^ . pk^_b) + e_b (+ Delta*p at coefficient 0 of c0)
-// pk^_b already carries the 1/N of the inverse transform. With KEEP_VHAT the transform of v
-// stays in registers for both products (3 transforms per limb); without it (N = 2^14,
-// register budget) it is recomputed (4 per limb). The first forward stage multiplies by a
-// ternary operand and needs no product.
+// Operands of fresh encryption: the public key modulo the auxiliary primes, transformed. Unit u
+// is a (limb l, prime i) pair (EncLimb::unit + i); block u writes
+//   NTT_{p_i}(pk_b, centered modulo q_l) * (N^{-1} (M_l / p_i)^{-1} 2^32) mod p_i
+// for both polynomials b, so that the Montgomery product with NTT(v) and the inverse transform
+// leave the CRT digit [v pk_b (M_l / p_i)^{-1}] mod p_i. Set-up code, one launch per key.
 // ---------------------------------------------------------------------------------------
-
-// Shared memory of one encryption block: the transform buffers (N words each; two where both
-// inverse transforms of a limb run in lockstep: N = 2^13, 8 residues per thread), v, e0, e1 as
-// int8 (3N bytes; two sets up to N = 2^13, used by alternate ciphertexts of the block), then the
-// search copy of the Gaussian table (32 words).
 template <int LOGN>
-static constexpr int kEncBufs = LOGN == 13 ? 2 : 1;
-
-template <int LOGN>
-static constexpr int kEncSampleSets = LOGN <= 13 ? 2 : 1;
-
-template <int LOGN>
-__device__ __forceinline__ u64* enc_cdt_smem(u64* smem)
+__global__ void __launch_bounds__(EncShape<LOGN>::T) k_pk_aux(const __grid_constant__ PkAuxArgs a)
 {
-    return smem + kEncBufs<LOGN> * (1 << LOGN) + ((3 * kEncSampleSets<LOGN>) << LOGN) / 8;
+    constexpr int N = 1 << LOGN, E = EncShape<LOGN>::E, LAST = NttShape<LOGN, E>::LAST;
+    extern __shared__ u64 smem[];
+    const int tid = threadIdx.x;
+    int l = 0;
+    while (l + 1 < a.L && (int)blockIdx.x >= a.unit[l + 1]) ++l;
+    const int u = blockIdx.x, i = u - a.unit[l];
+    const u64 q = a.q[l];
+    const u32 p = a.aux.p[i], k = a.k[u];
+    for (int b = 0; b < 2; ++b) {
+        const u64* src = a.pk + ((size_t)b * a.L + l) * N;
+        u32 r[1][E];
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const u64 c = src[elem_index<LOGN, 0, E>(tid, e)];
+            const u32 m = (u32)((c > q / 2 ? q - c : c) % p);
+            r[0][e] = c > q / 2 && m != 0 ? p - m : m;
+        }
+        ntt32_fwd<LOGN, 1, E, false>(reinterpret_cast<u32*>(smem), r, tid, a.aux.tw[i], p);
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            a.out[enc_pk_at<LOGN>(u, b, elem_index<LOGN, LAST, E>(tid, e))] = (u32)((u64)(r[0][e] % p) * k % p);
+    }
 }
 
 template <int LOGN>
-static constexpr size_t kEncSmem = ((sizeof(u64) * kEncBufs<LOGN> + 3 * kEncSampleSets<LOGN>) << LOGN) + 32 * sizeof(u64);
-
-// `it` counts the ciphertexts the block has encrypted before this one. With two sample sets the
-// block draws this ciphertext's samples into set it % 2 while slower warps may still read the
-// previous ciphertext's set in its last epilogue; the barrier after the sampling of the previous
-// ciphertext ordered every read of this set (two ciphertexts back) before it. With one set a
-// barrier must precede the sampling. The transform buffers need none (see the limb loop).
-template <int LOGN, bool KEEP_VHAT, int E>
-__device__ __forceinline__ void encrypt_ct(const EncArgs& a, int p, u64 seed, u64 id, u64* ct, u64* smem, int it)
+static cudaError_t pk_aux_launch(const PkAuxArgs& a, int n_units, cudaStream_t st)
 {
-    constexpr int N = 1 << LOGN;
-    constexpr int T = NttShape<LOGN, E>::T;
-    constexpr int LAST = NttShape<LOGN, E>::LAST;
-    constexpr int NB = kEncBufs<LOGN>;
-    int8_t* sv = reinterpret_cast<int8_t*>(smem + NB * N) + (kEncSampleSets<LOGN> == 2 ? (it & 1) * 3 * N : 0);
-    int8_t* se0 = sv + N;
-    int8_t* se1 = se0 + N;
-    const u64* tcdt = enc_cdt_smem<LOGN>(smem);   // filled by the kernel before its first ciphertext
+    const size_t smem = sizeof(u32) << LOGN;
+    cudaError_t e = cudaFuncSetAttribute(k_pk_aux<LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    k_pk_aux<LOGN><<<n_units, EncShape<LOGN>::T, smem, st>>>(a);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_pk_aux(const PkAuxArgs& a, int logn, int n_units, cudaStream_t st)
+{
+    switch (logn) {
+    case 10: return pk_aux_launch<10>(a, n_units, st);
+    case 11: return pk_aux_launch<11>(a, n_units, st);
+    case 12: return pk_aux_launch<12>(a, n_units, st);
+    case 13: return pk_aux_launch<13>(a, n_units, st);
+    case 14: return pk_aux_launch<14>(a, n_units, st);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+// ---------------------------------------------------------------------------------------
+// Fused fresh encryption (Sec. 2.2.2, with the library sign convention pk = (-a*s + e, a),
+// since the printed formulas do not cancel): one thread block per ciphertext.
+//   sample v (ternary), e0, e1 (Gaussian) once into shared memory; v^_i = NTT(v) modulo each
+//   auxiliary prime p_i once; then per limb l: c_b = [v pk_b] mod q_l + e_b (+ Delta*p at
+//   coefficient 0 of c0).
+// The product v pk_b is taken over the integers (pk_b centered, |coefficient| <= N q_l / 2) from
+// its residues modulo the limb's first np primes: y_i = INTT(v^_i . pk^_{b,i}) are the CRT digits
+// (the key operands carry 1/N and (M/p_i)^{-1}), and x = sum_i y_i M/p_i - k M with
+// k = round(sum_i y_i / p_i) is reduced modulo q_l by one 32-bit quotient estimate (enc_crt).
+// Three 64-bit transforms per limb become three 28-bit ones per ciphertext and four or six per limb
+// (19 at N = 2^13 with primes 60/40/60), at about a fifth of the multiply-pipe time each. Measured
+// against the 64-bit form: 4096 pixels at N = 2^13 3.03 -> 2.56 ms, 851 pixels at N = 2^14 and five
+// limbs 3.34 -> 1.77 ms, 1224 pixels at N = 2^12 0.66 -> 0.39 ms (there also more than one block per
+// SM). Bound by the integer multiply pipe (75 % busy), then by the exchanges between the passes.
+// ---------------------------------------------------------------------------------------
+
+// The sample word of a coefficient: v + 1 (bits 0-1), e0 + 32 (bits 2-7), e1 + 32 (bits 8-13).
+__device__ __forceinline__ u32 enc_sample(int v, int e0, int e1)
+{
+    return (u32)(v + 1) | ((u32)(e0 + 32) << 2) | ((u32)(e1 + 32) << 8);
+}
+
+// A limb's residue of one coefficient from its CRT digits (y[np - 1] the last prime's), noise added
+// (e_biased = e + 32): in [0, q). With k = round(sum y_i / p_i) the last digit less k times its
+// prime makes sum y_i M/p_i the product itself; it is offset by 5 primes to stay positive, which
+// lm.c0 takes back. The digits then sum to less than 2^30.6, so their products with the low and high
+// words of M/p_i mod q add up in 64 bits each. Primes of at most 32 bits (SMALL) have no high words.
+template <int NPR, bool SMALL>
+__device__ __forceinline__ u64 enc_crt(const EncLimb& lm, u32 y0, u32 y1, u32 y2, u32 e_biased)
+{
+    u32 sum = y0 + y1;
+    if constexpr (NPR == 3) sum += y2;
+    const u32 k = (sum + (1u << (kAuxBits - 1))) >> kAuxBits;
+    const u32 last = (NPR == 3 ? y2 : y1) + (5u - k) * lm.p_last;
+    u64 lo = (lm.c0 + e_biased) + (u64)y0 * lm.ml[0];
+    if constexpr (NPR == 3) lo += (u64)y1 * lm.ml[1];
+    lo += (u64)last * lm.ml[NPR - 1];
+    u32 T;   // floor(V / 2^(bits - 1)) < 2^32; the estimated quotient is short by less than 2.75
+    if constexpr (SMALL) {
+        T = (u32)(lo >> lm.t);
+    } else {
+        u64 hi = (u64)y0 * lm.mh[0];
+        if constexpr (NPR == 3) hi += (u64)y1 * lm.mh[1];
+        hi += (u64)last * lm.mh[NPR - 1];
+        T = (u32)((hi + (lo >> 32)) >> lm.t);
+        lo += hi << 32;
+    }
+    const u32 qhat = __umulhi(T, lm.mu);
+    lo += (u64)qhat * lm.nq_lo;             // less qhat q modulo 2^64: [0, 2.75 q)
+    lo += (u64)(qhat * lm.nq_hi) << 32;
+    return csub_s(csub_s(lo, 2 * lm.q), lm.q);
+}
+
+template <int LOGN>
+__device__ __forceinline__ void encrypt_ct(const EncArgs& a, int p, u64 seed, u64 id, u64* ct, u64* smem)
+{
+    using S = EncShape<LOGN>;
+    constexpr int N = 1 << LOGN, E = S::E, T = S::T, NP = S::NP, LAST = NttShape<LOGN, E>::LAST;
+    u32* ex = reinterpret_cast<u32*>(smem);                       // exchange buffer, N words of 4 NP bytes
+    u32* vh = ex + NP * N;                                        // v^ modulo S::KEEP primes, thread-major
+    uint16_t* smp = reinterpret_cast<uint16_t*>(vh + S::KEEP * N);
+    const u64* tcdt = reinterpret_cast<const u64*>(reinterpret_cast<unsigned char*>(smem) + S::CDT_AT);
     const int tid = threadIdx.x;
     const int L = a.L;
-    if constexpr (kEncSampleSets<LOGN> == 1) __syncthreads();   // the previous ciphertext's samples no longer read
-    for (int b = tid; b < N / 4; b += T) {
-        Words4 w = philox(seed, kStreamV, id, (u32)b);
-        u32 packed = 0;
+    __syncthreads();   // the previous ciphertext's samples no longer read
+    for (int b = tid; b < N / 4; b += T) {         // coefficients 4b .. 4b + 3
+        const Words4 wv = philox(seed, kStreamV, id, (u32)b);
+        u32 packed[2];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) packed |= ((u32)(uint8_t)(int8_t)ternary_of(w.w[i])) << (8 * i);
-        reinterpret_cast<u32*>(sv)[b] = packed;
+        for (int h = 0; h < 2; ++h) {
+            const Words4 w0 = philox(seed, kStreamE0, id, (u32)(2 * b + h));
+            const Words4 w1 = philox(seed, kStreamE1, id, (u32)(2 * b + h));
+            const u32 lo = enc_sample(ternary_of(wv.w[2 * h]), gauss_of_sorted((u64)w0.w[0] | ((u64)w0.w[1] << 32), tcdt),
+                                      gauss_of_sorted((u64)w1.w[0] | ((u64)w1.w[1] << 32), tcdt));
+            const u32 hi = enc_sample(ternary_of(wv.w[2 * h + 1]),
+                                      gauss_of_sorted((u64)w0.w[2] | ((u64)w0.w[3] << 32), tcdt),
+                                      gauss_of_sorted((u64)w1.w[2] | ((u64)w1.w[3] << 32), tcdt));
+            packed[h] = lo | (hi << 16);
+        }
+        reinterpret_cast<uint2*>(smp)[b] = make_uint2(packed[0], packed[1]);
     }
-    for (int b = tid; b < N / 2; b += T) {
-        Words4 w0 = philox(seed, kStreamE0, id, (u32)b);
-        Words4 w1 = philox(seed, kStreamE1, id, (u32)b);
-        int g00 = gauss_of_sorted((u64)w0.w[0] | ((u64)w0.w[1] << 32), tcdt);
-        int g01 = gauss_of_sorted((u64)w0.w[2] | ((u64)w0.w[3] << 32), tcdt);
-        int g10 = gauss_of_sorted((u64)w1.w[0] | ((u64)w1.w[1] << 32), tcdt);
-        int g11 = gauss_of_sorted((u64)w1.w[2] | ((u64)w1.w[3] << 32), tcdt);
-        reinterpret_cast<uint16_t*>(se0)[b] = (uint16_t)((uint8_t)g00 | ((uint16_t)(uint8_t)g01 << 8));
-        reinterpret_cast<uint16_t*>(se1)[b] = (uint16_t)((uint8_t)g10 | ((uint16_t)(uint8_t)g11 << 8));
-    }
-    __syncthreads();
 
     const int x0 = elem_index<LOGN, 0, E>(tid, 0);       // first-pass layout: x0 + elem_offset(e)
     const int xl = elem_index<LOGN, LAST, E>(tid, 0);    // last-pass layout
-    if constexpr (NB == 2 && KEEP_VHAT) {
-        // per limb: v^ = NTT(v), both products v^ . pk^_b at once, then the two inverse
-        // transforms in lockstep (one pass structure, barriers and twiddle loads shared). No
-        // block barrier separates the transforms: a transform's first exchange stores to the
-        // slots of the layout the previous one last loaded (pass 0 after an inverse, the last
-        // pass after a forward), so every thread overwrites only slots it has read itself, and
-        // the second buffer's last readers (the previous limb's inverse) are behind the forward
-        // transform's block-wide exchanges (3.19 -> 3.10 ms).
-        for (int l = 0; l < L; ++l) {
-            const u64 q = a.rns.q[l];
-            const ModTables t = a.rns.tab[l];
-            u64 r[1][E];
+    // First the third prime, for the limbs that need it: its digits wait in the output's own words
+    // (each thread's coefficients of the ciphertext, which it overwrites with the residues below),
+    // so that at most two primes' digits are in registers. Then the first two primes of every limb.
+#pragma unroll 1
+    for (int phase = a.aux.n == 3 ? 0 : 1; phase < 2; ++phase) {
+        const int i0 = phase == 0 ? 2 : 0, i1 = phase == 0 ? 3 : 2;
+#pragma unroll 1
+        for (int i = i0; i < i1; ++i) {
+            __syncthreads();   // the exchange buffer's last readers are done
+            u32 r[1][E];
 #pragma unroll
-            for (int e = 0; e < E; ++e) r[0][e] = small_mod(sv[x0 + elem_offset<LOGN, 0, E>(e)], q);
-            ntt_fwd_regs<LOGN, 1, true, false, E>(smem, r, tid, t, q);
-            u64 rr[2][E];
-            const ulonglong2* pk0 = a.pk_pair + (size_t)l * N + xl;
-            const ulonglong2* pk1 = a.pk_pair + ((size_t)L + l) * N + xl;
+            for (int e = 0; e < E; ++e) r[0][e] = (u32)((int)(smp[x0 + elem_offset<LOGN, 0, E>(e)] & 3u) - 1);
+            ntt32_fwd<LOGN, 1, E, true>(ex, r, tid, a.aux.tw[i], a.aux.p[i]);
 #pragma unroll
-            for (int e = 0; e < E; ++e) {
-                const ulonglong2 w0 = __ldg(pk0 + elem_offset<LOGN, LAST, E>(e));
-                const ulonglong2 w1 = __ldg(pk1 + elem_offset<LOGN, LAST, E>(e));
-                rr[0][e] = shoup_lazy(r[0][e], w0.x, w0.y, q);
-                rr[1][e] = shoup_lazy(r[0][e], w1.x, w1.y, q);
-            }
-            ntt_inv_regs<LOGN, 2, false, E>(smem, rr, tid, t, q);
-#pragma unroll
-            for (int pb = 0; pb < 2; ++pb) {
-                const int8_t* noise = (pb == 0 ? se0 : se1) + x0;
-                u64* dst = ct + ((u64)pb * L + l) * N + x0;
-#pragma unroll
-                for (int e = 0; e < E; ++e) {
-                    const int x = elem_offset<LOGN, 0, E>(e);
-                    u64 v = rr[pb][e] + (q + (u64)(i64)noise[x]);   // [q - 31, 3q + 31)
-                    v = csub(csub(v, 2 * q), q);
-                    if (pb == 0 && x == 0 && x0 == 0) v = add_mod(v, a.dm[l * 256 + p], q);   // coefficient 0
-                    __stcs(dst + x, v);
-                }
-            }
+            for (int e = 0; e < E; ++e) vh[(i - i0) * N + e * T + tid] = r[0][e];
         }
-        return;
-    }
-    // one transform at a time: a block barrier is needed only between two inverse transforms
-    // (with v^ kept, the second product's), as in the lockstep form above
-    for (int l = 0; l < L; ++l) {
-        const u64 q = a.rns.q[l];
-        const ModTables t = a.rns.tab[l];
-        u64 r[1][E];
-        u64 vh[KEEP_VHAT ? E : 1];
-        for (int pb = 0; pb < 2; ++pb) {
-            if (KEEP_VHAT && pb == 1) {
+#pragma unroll 1
+        for (int l = 0; l < L; ++l) {
+            const EncLimb& lm = a.limb[l];
+            if (i0 >= lm.np) continue;
+#pragma unroll 1
+            for (int pb = 0; pb < 2; pb += NP) {
+                u32 ya[NP][E], y[NP][E];   // digits modulo the first prime, and the current one
+#pragma unroll 1
+                for (int i = i0; i < i1; ++i) {
+                    const u32 pi = a.aux.p[i], pinv = a.aux.pinv[i];
+                    const u32* pk = a.pk_aux + enc_pk_at<LOGN>(lm.unit + i, pb, xl);
 #pragma unroll
-                for (int e = 0; e < E; ++e) r[0][e] = vh[KEEP_VHAT ? e : 0];
-            } else {
+                    for (int e = 0; e < E; ++e) {
+                        if (i == 1) {
 #pragma unroll
-                for (int e = 0; e < E; ++e) r[0][e] = small_mod(sv[x0 + elem_offset<LOGN, 0, E>(e)], q);
-                ntt_fwd_regs<LOGN, 1, true, false, E>(smem, r, tid, t, q);   // after an inverse: no barrier
-                if constexpr (KEEP_VHAT) {
-#pragma unroll
-                    for (int e = 0; e < E; ++e) vh[e] = r[0][e];
+                            for (int n = 0; n < NP; ++n) ya[n][e] = y[n][e];
+                        }
+                        const u32 v = vh[(i - i0) * N + e * T + tid];
+                        const int o = elem_offset<LOGN, LAST, E>(e);
+                        if constexpr (NP == 2) {
+                            const uint2 w = __ldg(reinterpret_cast<const uint2*>(pk) + o);
+                            y[0][e] = mont32(v, w.x, pi, pinv);
+                            y[NP - 1][e] = mont32(v, w.y, pi, pinv);
+                        } else {
+                            y[0][e] = mont32(v, __ldg(pk + o), pi, pinv);
+                        }
+                    }
+                    __syncthreads();
+                    ntt32_inv<LOGN, NP, E>(ex, y, tid, a.aux.itw[i], pi);
                 }
-            }
-            const ulonglong2* pk = a.pk_pair + ((size_t)pb * L + l) * N + xl;
+                u64* dst = ct + ((u64)pb * L + l) * N + x0;
+                if (phase == 0) {
 #pragma unroll
-            for (int e = 0; e < E; ++e) {
-                const ulonglong2 w = __ldg(pk + elem_offset<LOGN, LAST, E>(e));
-                r[0][e] = shoup_lazy(r[0][e], w.x, w.y, q);
-            }
-            if (KEEP_VHAT && pb == 1) __syncthreads();   // an inverse right after an inverse
-            ntt_inv_regs<LOGN, 1, false, E>(smem, r, tid, t, q);
-            const int8_t* noise = (pb == 0 ? se0 : se1) + x0;
-            u64* dst = ct + ((u64)pb * L + l) * N + x0;
+                    for (int n = 0; n < NP; ++n)
 #pragma unroll
-            for (int e = 0; e < E; ++e) {
-                const int x = elem_offset<LOGN, 0, E>(e);
-                u64 v = r[0][e] + (q + (u64)(i64)noise[x]);   // [q - 31, 3q + 31)
-                v = csub(csub(v, 2 * q), q);
-                if (pb == 0 && x == 0 && x0 == 0) v = add_mod(v, a.dm[l * 256 + p], q);   // coefficient 0
-                __stcs(dst + x, v);
+                        for (int e = 0; e < E; ++e)
+                            dst[(u64)n * L * N + elem_offset<LOGN, 0, E>(e)] = y[n][e];
+                    continue;
+                }
+                auto write = [&](auto residue) {
+#pragma unroll
+                    for (int n = 0; n < NP; ++n)
+#pragma unroll
+                        for (int e = 0; e < E; ++e) {
+                            const int x = elem_offset<LOGN, 0, E>(e);
+                            u64* o = dst + (u64)n * L * N + x;
+                            const u32 s = smp[x0 + x];
+                            u64 v = residue(n, e, o, pb + n == 0 ? (s >> 2) & 63u : s >> 8);
+                            if (pb + n == 0 && x == 0 && x0 == 0) v = add_mod(v, a.dm[l * 256 + p], lm.q);   // coefficient 0
+                            __stcs(o, v);
+                        }
+                };
+                if (lm.np == 3)
+                    write([&](int n, int e, const u64* o, u32 eb) {
+                        return enc_crt<3, false>(lm, ya[n][e], y[n][e], (u32)*o, eb);
+                    });
+                else if (lm.bits > 32)
+                    write([&](int n, int e, const u64*, u32 eb) { return enc_crt<2, false>(lm, ya[n][e], y[n][e], 0, eb); });
+                else
+                    write([&](int n, int e, const u64*, u32 eb) { return enc_crt<2, true>(lm, ya[n][e], y[n][e], 0, eb); });
             }
         }
     }
 }
 
-template <int LOGN, bool KEEP_VHAT, int E>
-__global__ void __launch_bounds__(NttShape<LOGN, E>::T, 1) k_encrypt_fresh(const __grid_constant__ EncArgs a)
+template <int LOGN>
+__device__ __forceinline__ void encrypt_setup(const EncArgs& a, u64* smem)
+{
+    cdt_for_search(a.cdt, reinterpret_cast<u64*>(reinterpret_cast<unsigned char*>(smem) + EncShape<LOGN>::CDT_AT));
+    __syncthreads();
+}
+
+template <int LOGN>
+__global__ void __launch_bounds__(EncShape<LOGN>::T, EncShape<LOGN>::BLOCKS)
+    k_encrypt_fresh(const __grid_constant__ EncArgs a)
 {
     extern __shared__ u64 smem[];
-    cdt_for_search(a.cdt, enc_cdt_smem<LOGN>(smem));
-    __syncthreads();
+    encrypt_setup<LOGN>(a, smem);
     const u64 ct_len = (u64)2 * a.L << LOGN;
-    int it = 0;
     // all pixels, or a listed subset (the misses of a value cache) shared evenly; one call site,
     // so the kernel holds one copy of the transform code
     const u64 n = a.idx != nullptr ? (u64)*a.n_idx : a.n_ct;
@@ -406,76 +494,62 @@ __global__ void __launch_bounds__(NttShape<LOGN, E>::T, 1) k_encrypt_fresh(const
         const u64 k = a.idx != nullptr ? (u64)a.idx[g] : g;
         const int p = a.pixels[k];
         if (a.skip_lut != nullptr && a.skip_lut[p] >= 0) continue;  // uniform across the block
-        encrypt_ct<LOGN, KEEP_VHAT, E>(a, p, a.seed, a.id_base + k, a.out + k * ct_len, smem, it++);
+        encrypt_ct<LOGN>(a, p, a.seed, a.id_base + k, a.out + k * ct_len, smem);
     }
 }
 
-template <int LOGN, bool KEEP_VHAT, int E>
-__global__ void __launch_bounds__(NttShape<LOGN, E>::T, 1) k_encrypt_fresh_batch(const __grid_constant__ EncArgs a,
-                                                                              const __grid_constant__ SegTable t)
+template <int LOGN>
+__global__ void __launch_bounds__(EncShape<LOGN>::T, EncShape<LOGN>::BLOCKS)
+    k_encrypt_fresh_batch(const __grid_constant__ EncArgs a, const __grid_constant__ SegTable t)
 {
     extern __shared__ u64 smem[];
-    cdt_for_search(a.cdt, enc_cdt_smem<LOGN>(smem));
-    __syncthreads();
+    encrypt_setup<LOGN>(a, smem);
     const u64 ct_len = (u64)2 * a.L << LOGN;
     const u64 total = t.start[t.n];
-    int it = 0;
     for (u64 g = blockIdx.x; g < total; g += gridDim.x) {
         const int s = seg_of(t, g);
         const u64 k = g - t.start[s];
         const int p = t.px[s][k];
         if (a.skip_lut != nullptr && a.skip_lut[p] >= 0) continue;
-        encrypt_ct<LOGN, KEEP_VHAT, E>(a, p, t.seed[s], k, t.out[s] + k * ct_len, smem, it++);
+        encrypt_ct<LOGN>(a, p, t.seed[s], k, t.out[s] + k * ct_len, smem);
     }
 }
 
-// Residues per thread of the encryption transforms: 8 at N = 2^13 (1024 threads, twice the
-// warps per SM of the 16-residue layout), else 16.
+// Persistent grid: the blocks that fit on the GPU at once, each walking its share of the
+// ciphertexts. With pixels to skip in-kernel the shares would be uneven, so there more blocks than
+// fit are launched.
 template <int LOGN>
-static constexpr int kEncE = LOGN == 13 ? 8 : 16;
+static unsigned enc_grid(u64 n, int num_sms, bool skips)
+{
+    const u64 cap = (u64)num_sms * EncShape<LOGN>::BLOCKS * (skips ? 16 : 1);
+    return (unsigned)(n < cap ? n : cap);
+}
 
 template <int LOGN>
 static cudaError_t enc_launch(const EncArgs& a, cudaStream_t st)
 {
-    constexpr bool keep = LOGN <= 13;
-    constexpr int E = kEncE<LOGN>;
-    const int T = NttShape<LOGN, E>::T;
-    const size_t smem = kEncSmem<LOGN>;
-    cudaError_t e = cudaFuncSetAttribute(k_encrypt_fresh<LOGN, keep, E>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
+    using S = EncShape<LOGN>;
+    cudaError_t e = cudaFuncSetAttribute(k_encrypt_fresh<LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
     if (e != cudaSuccess) return e;
-    // persistent: one block per SM (the shared memory fits one), each walking its share of the
-    // ciphertexts, so a block's sampling overlaps its previous ciphertext's epilogue (3.10 ->
-    // 3.06 ms); a listed subset is shared the same way. With pixels to skip in-kernel the shares
-    // would be uneven, so there every ciphertext is a block of its own (a static share of the
-    // whole image: 2.40 -> 2.81 ms for the misses of the top-32 cache).
-    const u64 cap = a.skip_lut == nullptr && a.num_sms > 0 ? (u64)a.num_sms : (u64)(1u << 30);
-    const u64 grid = a.n_ct < cap ? a.n_ct : cap;
-    k_encrypt_fresh<LOGN, keep, E><<<(unsigned)grid, T, smem, st>>>(a);
+    k_encrypt_fresh<LOGN><<<enc_grid<LOGN>(a.n_ct, a.num_sms, a.skip_lut != nullptr), S::T, S::SMEM, st>>>(a);
     return cudaGetLastError();
 }
 
 template <int LOGN>
 static cudaError_t enc_batch_launch(const EncArgs& a, const SegTable& t, int num_sms, cudaStream_t st)
 {
-    constexpr bool keep = LOGN <= 13;
-    constexpr int E = kEncE<LOGN>;
-    const int T = NttShape<LOGN, E>::T;
-    const size_t smem = kEncSmem<LOGN>;
-    cudaError_t e = cudaFuncSetAttribute(k_encrypt_fresh_batch<LOGN, keep, E>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    using S = EncShape<LOGN>;
+    cudaError_t e = cudaFuncSetAttribute(k_encrypt_fresh_batch<LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)S::SMEM);
     if (e != cudaSuccess) return e;
-    const u64 total = t.start[t.n];
-    const u64 cap = (u64)num_sms * 4;   // persistent: a few resident blocks per SM
-    const unsigned grid = (unsigned)(total < cap ? total : cap);
-    k_encrypt_fresh_batch<LOGN, keep, E><<<grid, T, smem, st>>>(a, t);
+    k_encrypt_fresh_batch<LOGN><<<enc_grid<LOGN>(t.start[t.n], num_sms, a.skip_lut != nullptr), S::T, S::SMEM, st>>>(a, t);
     return cudaGetLastError();
 }
 
 cudaError_t launch_encrypt_fresh_batch(const EncArgs& a, const SegTable& t, int num_sms, cudaStream_t st)
 {
     if (t.n <= 0 || t.start[t.n] == 0) return cudaSuccess;
-    switch (a.rns.logn) {
+    switch (a.logn) {
     case 10: return enc_batch_launch<10>(a, t, num_sms, st);
     case 11: return enc_batch_launch<11>(a, t, num_sms, st);
     case 12: return enc_batch_launch<12>(a, t, num_sms, st);
@@ -503,7 +577,7 @@ cudaError_t launch_miss_list(const uint8_t* px, u64 n, const int32_t* lut, u32* 
 cudaError_t launch_encrypt_fresh(const EncArgs& a, cudaStream_t st)
 {
     if (a.n_ct == 0) return cudaSuccess;
-    switch (a.rns.logn) {
+    switch (a.logn) {
     case 10: return enc_launch<10>(a, st);
     case 11: return enc_launch<11>(a, st);
     case 12: return enc_launch<12>(a, st);

@@ -48,6 +48,7 @@ __host__ __device__ constexpr int swz(int x)
 template <int LOGN, int S0, int E = 16>
 struct Pass {
     static constexpr int LE = Radix<E>::LE;
+    static constexpr int R = E;                                      // residues per thread
     static constexpr int N = 1 << LOGN;
     static constexpr int T = N / E;
     static constexpr int S = (LOGN - S0) < LE ? (LOGN - S0) : LE;  // stages in this pass
