@@ -30,6 +30,16 @@ __device__ __forceinline__ u64 shoup_lazy(u64 x, u64 w, u64 wp, u64 q)
     return x * w - hi * q;
 }
 
+// The same in [0, 4q) with three 32-bit products for the quotient instead of four: the low words'
+// product and the fractions of the cross products are dropped, so the quotient is short by at most
+// two.
+__host__ __device__ __forceinline__ u64 shoup3(u64 x, u64 w, u64 wp, u64 q)
+{
+    const u32 xl = (u32)x, xh = (u32)(x >> 32), pl = (u32)wp, ph = (u32)(wp >> 32);
+    const u64 hi = (u64)xh * ph + (((u64)xh * pl) >> 32) + (((u64)xl * ph) >> 32);
+    return x * w - hi * q;
+}
+
 __device__ __forceinline__ u64 shoup(u64 x, u64 w, u64 wp, u64 q)
 {
     u64 r = shoup_lazy(x, w, wp, q);
@@ -38,7 +48,7 @@ __device__ __forceinline__ u64 shoup(u64 x, u64 w, u64 wp, u64 q)
 
 __device__ __forceinline__ u64 csub(u64 x, u64 q) { return x >= q ? x - q : x; }
 
-// The same for x, q < 2^63: the sign of the difference decides, one comparison of high words.
+// The same for q <= 2^63 and x < q + 2^63: the sign of the difference decides (one comparison).
 __device__ __forceinline__ u64 csub_s(u64 x, u64 q)
 {
     const i64 d = (i64)(x - q);
@@ -76,17 +86,25 @@ __device__ __forceinline__ u64 mul_mod(u64 a, u64 b, u64 q, u64 m0, u64 m1)
     return r;
 }
 
-// Montgomery product a*b*2^{-64} mod q for a, b < q < 2^62, q odd, qinv = -q^{-1} mod 2^64
-// (Montgomery, Math. Comp. 44, 1985): with m = (ab mod 2^64) * qinv mod 2^64, ab + mq is a
-// multiple of 2^64 and (ab + mq) / 2^64 < 2q. The low words of ab and mq sum to 0 or 2^64, so
-// the carry into the high word is (ab mod 2^64 != 0). Callers fold the factor 2^64 into a
-// constant applied later.
-__device__ __forceinline__ u64 mont_mul(u64 a, u64 b, u64 q, u64 qinv)
+// Montgomery product a*b*2^{-64} mod q, q odd, in two steps of 32 bits (Montgomery, Math. Comp. 44,
+// 1985): adding m q with m = (t mod 2^32) (-q^{-1}) makes the low word of t vanish. The result is
+// below a b / 2^64 + q: in [0, 2q) for a, b < 4q with q < 2^60, or for a, b < 62q with q < 2^50.
+// qinv = -q^{-1} mod 2^64 (its low word is used). Callers fold the factor 2^64 into a constant
+// applied later. Ten 32-bit products; with 64-bit words it took sixteen.
+__host__ __device__ __forceinline__ u64 mont_lazy(u64 a, u64 b, u64 q, u64 qinv)
 {
-    const u64 lo = a * b;
-    const u64 m = lo * qinv;
-    const u64 t = mulhi(a, b) + mulhi(m, q) + (lo != 0 ? 1 : 0);
-    return csub(t, q);
+    const u32 a0 = (u32)a, a1 = (u32)(a >> 32), b0 = (u32)b, b1 = (u32)(b >> 32);
+    const u32 q0 = (u32)q, q1 = (u32)(q >> 32), qi = (u32)qinv;
+    const u64 p = (u64)a0 * b0;
+    const u64 r = (u64)a0 * b1 + (p >> 32);
+    const u64 s = (u64)a1 * b0 + (u32)r;
+    const u64 u = (u64)a1 * b1 + (r >> 32) + (s >> 32);        // words 2 and 3 of a b; word 1 is s's low
+    const u32 m = (u32)p * qi;
+    const u64 v = (u64)m * q0 + (u32)p;
+    const u64 w = (u64)m * q1 + (u32)s + (v >> 32);
+    const u32 m2 = (u32)w * qi;
+    const u64 v2 = (u64)m2 * q0 + (u32)w;
+    return (u64)m2 * q1 + u + (w >> 32) + (v2 >> 32);
 }
 
 // --------------------------------------------------------------------------------------

@@ -1257,15 +1257,16 @@ extern "C" ichee_status ichee_meanfilter_rows(ichee_ctx* c, const uint64_t* d_in
 // entry point and the split form (ichee_sqdiff_accumulate / ichee_sqdiff_finish); they differ
 // only in where the working memory comes from.
 
-// Accumulating blocks of the first step: one per SM, rounded down to a multiple of the limbs
-// (of twice the limbs in the split form), and the scratch words of one block's slice.
+// Accumulating blocks of the first step: as many as the SMs hold, but no more than there are
+// (pair, limb) items, in multiples of the limbs (of twice the limbs in the split form), and the
+// scratch words of one block's slice.
 static int sqdiff_unit(const ichee_ctx* c, int limbs) { return sqdiff_split(c->logn) ? 2 * limbs : limbs; }
 
-static int sqdiff_blocks(const ichee_ctx* c, int limbs)
+static int sqdiff_blocks(const ichee_ctx* c, int limbs, u64 n_ct)
 {
     const int u = sqdiff_unit(c, limbs);
-    const int nb = (c->num_sms / u) * u;
-    return nb < u ? u : nb;
+    const u64 groups = std::max<u64>(1, (u64)c->num_sms * sqdiff_blocks_per_sm(c->logn) / u);
+    return (int)std::min<u64>(groups, n_ct) * u;
 }
 
 static size_t sqdiff_slice_words(const ichee_ctx* c) { return (size_t)(sqdiff_split(c->logn) ? 2 : 4) * c->n; }
@@ -1373,7 +1374,7 @@ static ichee_status op_sqdiff(ichee_ctx* c, const uint64_t* d_a, const ichee_cti
     if (!c->have_evk) return fail(ICHEE_EUNSUPPORTED, "matching needs the evaluation key (ICHEE_WITH_EVK)");
     if (ma->level == 0) return fail(ICHEE_ELEVEL, "matching needs a limb to drop");
     const int limbs = (int)ma->level + 1;
-    const int n_blocks = sqdiff_blocks(c, limbs);
+    const int n_blocks = sqdiff_blocks(c, limbs, (u64)ma->h * ma->w * ma->c);
     const size_t words = relin_words(c, limbs) + (size_t)n_blocks * sqdiff_slice_words(c);
     CK(c->scratch.ensure(words * 8, c->user_alloc, c->user_free, c->user_alloc_ctx, st));
     return sqdiff_in(c, d_a, ma, d_b, (u64*)c->scratch.p, n_blocks, d_out, mout, st);
@@ -1418,7 +1419,7 @@ extern "C" ichee_status ichee_sqdiff_accumulate(ichee_ctx* c, const uint64_t* d_
     s = check_span(d_acc, acc_words * 8, "accumulator");
     if (s != ICHEE_OK) return s;
     cudaStream_t st = (cudaStream_t)stream;
-    const int n_blocks = sqdiff_blocks(c, limbs);
+    const int n_blocks = sqdiff_blocks(c, limbs, (u64)ma->h * ma->w * ma->c);
     CK(c->scratch.ensure((size_t)n_blocks * sqdiff_slice_words(c) * 8, c->user_alloc, c->user_free, c->user_alloc_ctx,
                          st));
     return sqdiff_partial_sum(c, d_a, ma, d_b, (u64*)c->scratch.p, n_blocks, d_acc, accumulate != 0, st);
@@ -1667,7 +1668,7 @@ extern "C" ichee_status ichee_sqdiff_sum_noalloc(ichee_ctx* c, const uint64_t* d
     const size_t slice_w = sqdiff_slice_words(c);
     const size_t fit = fixed_w < cap_w ? (cap_w - fixed_w) / slice_w : 0;
     const int unit = sqdiff_unit(c, limbs);
-    int n_blocks = sqdiff_blocks(c, limbs);
+    int n_blocks = sqdiff_blocks(c, limbs, (u64)ma->h * ma->w * ma->c);
     if ((size_t)n_blocks > fit) n_blocks = (int)((fit / unit) * unit);
     if (n_blocks < unit)
         return fail(ICHEE_EINVAL, "matching at N=%zu with %d limbs needs %zu bytes of scratch; the allocation-free "

@@ -94,12 +94,12 @@ __global__ void __launch_bounds__(NttShape<LOGN>::T) k_ntt_fwd(const __grid_cons
     const int m = b.midx[blockIdx.x % b.nl];
     const u64 q = rns.q[m];
     u64* d = b.data + (size_t)blockIdx.x * (1 << LOGN);
-    u64 r[1][16];
+    u64 r[16];
 #pragma unroll
-    for (int e = 0; e < 16; ++e) r[0][e] = d[elem_index<LOGN, 0>(tid, e)];
-    ntt_fwd_regs<LOGN, 1>(sm, r, tid, rns.tab[m], q);
+    for (int e = 0; e < 16; ++e) r[e] = d[elem_index<LOGN, 0>(tid, e)];
+    ntt_fwd_regs<LOGN, false, 16, 8, 1>(sm, r, tid, rns.tab[m], q);
 #pragma unroll
-    for (int e = 0; e < 16; ++e) d[elem_index<LOGN, NttShape<LOGN>::LAST>(tid, e)] = csub(csub(r[0][e], 2 * q), q);
+    for (int e = 0; e < 16; ++e) d[elem_index<LOGN, NttShape<LOGN>::LAST>(tid, e)] = below1<8>(r[e], q);
 }
 
 template <int LOGN>
@@ -110,12 +110,12 @@ __global__ void __launch_bounds__(NttShape<LOGN>::T) k_ntt_inv(const __grid_cons
     const int m = b.midx[blockIdx.x % b.nl];
     const u64 q = rns.q[m];
     u64* d = b.data + (size_t)blockIdx.x * (1 << LOGN);
-    u64 r[1][16];
+    u64 r[16];
 #pragma unroll
-    for (int e = 0; e < 16; ++e) r[0][e] = d[elem_index<LOGN, NttShape<LOGN>::LAST>(tid, e)];
-    ntt_inv_regs<LOGN, 1>(sm, r, tid, rns.tab[m], q);
+    for (int e = 0; e < 16; ++e) r[e] = d[elem_index<LOGN, NttShape<LOGN>::LAST>(tid, e)];
+    ntt_inv_regs<LOGN, false, 16, 8>(sm, r, tid, rns.tab[m], q);
 #pragma unroll
-    for (int e = 0; e < 16; ++e) d[elem_index<LOGN, 0>(tid, e)] = csub(r[0][e], q);
+    for (int e = 0; e < 16; ++e) d[elem_index<LOGN, 0>(tid, e)] = below1<4>(r[e], q);
 }
 
 template <int LOGN>

@@ -6,23 +6,47 @@
 
 namespace ichee {
 
+// Moduli below this run their transforms without any fold: outputs stay below (6 + 4 * 14) q, as the
+// Montgomery products take them (mont_lazy).
+constexpr u64 kNoFoldBelow = 1ull << 50;
+
+// The tensor terms of two neighbouring positions added to the accumulators at acc, acc + n, acc + 2n
+// (in [0, 2q)): d0^2, d0 d1, d1^2, each carrying 2^{-64}, undone after the inverse transform.
+__device__ __forceinline__ void tensor_pair(u64* acc, int n, u64 d1x, u64 d1y, u64 d0x, u64 d0y, u64 q, u64 qinv)
+{
+    auto add = [&](u64* p, u64 tx, u64 ty) {
+        ulonglong2* s = reinterpret_cast<ulonglong2*>(p);
+        const ulonglong2 v = *s;
+        *s = make_ulonglong2(csub_s(v.x + tx, 2 * q), csub_s(v.y + ty, 2 * q));
+    };
+    add(acc, mont_lazy(d0x, d0x, q, qinv), mont_lazy(d0y, d0y, q, qinv));
+    add(acc + n, mont_lazy(d0x, d1x, q, qinv), mont_lazy(d0y, d1y, q, qinv));
+    add(acc + 2 * n, mont_lazy(d1x, d1x, q, qinv), mont_lazy(d1y, d1y, q, qinv));
+}
+
 // One block per SM-sized share of the work: block j owns limb l = j % limbs and every
 // (n_blocks/limbs)-th ciphertext. Per ciphertext it forms d = a - b for its limb, transforms
-// d0 and d1, and accumulates (d0^2, 2 d0 d1, d1^2) position by position into its own slice of
-// the scratch buffer (each position is owned by one thread, so no atomics are needed). The
-// transform of d0 waits in a second shared-memory buffer (SMEM_D0) or, for the 2^14 ring whose
-// buffers do not both fit, in the fourth scratch row; d1's waits in the transform buffer. Every
-// thread parks and reads back only the slots of its own last-pass registers -- the slots it
-// loaded in the transform's last exchange -- so no barrier follows the transform (2.69 -> 2.67
-// ms); the barrier before each transform remains (its first exchange writes other slots).
-template <int LOGN, bool SMEM_D0, int E>
-__global__ void __launch_bounds__(NttShape<LOGN, E>::T, 1) k_sqdiff_accumulate(const __grid_constant__ SqDiffArgs a)
+// d0 and d1, and accumulates (d0^2, d0 d1, d1^2) position by position into its own slice of
+// the scratch buffer (each position is owned by one thread, so no atomics are needed; the middle
+// term is doubled when the slices are added up). d0 is transformed and waits in one shared-memory
+// buffer, d1 in the other. Every thread parks and reads back only the slots of its own last-pass
+// registers -- the slots it loaded in the transform's last exchange -- so no barrier follows the
+// transform. Values stay lazily reduced throughout (ntt.cuh): the difference in [0, 2q), the
+// transforms' outputs below 4q as the Montgomery products take them, the accumulators in [0, 2q).
+// Moduli below 2^50 (NOFOLD) need no reduction inside a transform at all.
+// Whole matching calls against the earlier form (a conditional subtraction per butterfly, exact
+// quotients, canonical values, one block of 16 residues a thread per SM below N = 2^13): 4096 pairs
+// at N = 2^13 with primes 60/40/60 2.59 -> 2.31 ms, 3072 pairs at N = 2^14 and five limbs 6.99 -> 6.60
+// ms, 1600 pairs at N = 2^12 0.74 -> 0.55 ms. The multiply pipe is about half busy: transforms,
+// exchanges and twiddle loads of the one block per SM follow each other between its barriers.
+template <int LOGN, int E, int CAP>
+__device__ __forceinline__ void sqdiff_accumulate(const SqDiffArgs& a, u64* buf)
 {
     constexpr int N = 1 << LOGN;
     constexpr int LAST = NttShape<LOGN, E>::LAST;
-    extern __shared__ u64 buf[];
+    constexpr int OUT = fwd_out<LOGN, false, CAP, 2>();
     u64* acc = a.partial + (size_t)blockIdx.x * 4 * N;
-    u64* d0buf = SMEM_D0 ? buf + N : acc + 3 * N;
+    u64* d0buf = buf + N;
     const int tid = threadIdx.x;
     const int limbs = a.limbs;
     const int l = blockIdx.x % limbs;
@@ -48,52 +72,37 @@ __global__ void __launch_bounds__(NttShape<LOGN, E>::T, 1) k_sqdiff_accumulate(c
             const int x0 = elem_index<LOGN, 0, E>(tid, 0);   // first-pass layout: x0 + elem_offset(e)
             const u64* pa = A + ((u64)pb * limbs + l) * N + x0;
             const u64* pbb = B + ((u64)pb * limbs + l) * N + x0;
-            u64 r[1][E];
+            u64 r[E];
 #pragma unroll
             for (int e = 0; e < E; ++e) {
                 const int x = elem_offset<LOGN, 0, E>(e);
-                r[0][e] = sub_mod(__ldcs(pa + x), __ldcs(pbb + x), q);
+                r[e] = __ldcs(pa + x) + q - __ldcs(pbb + x);
             }
-            // with both buffers in shared memory d0 is transformed in its parking buffer and d1 in
-            // the other one: d1's transform then starts after d0's block-wide exchanges, which
-            // every thread reaches only after its reads of the previous pixel, so it needs no
-            // barrier of its own
-            if (pb == 0 || !SMEM_D0) __syncthreads();
-            ntt_fwd_regs<LOGN, 1, false, false, E>(SMEM_D0 && pb == 0 ? d0buf : buf, r, tid, t, q);
+            // d0 is transformed in its parking buffer and d1 in the other one: d1's transform then
+            // starts after d0's block-wide exchanges, which every thread reaches only after its
+            // reads of the previous pixel, so it needs no barrier of its own
+            if (pb == 0) __syncthreads();
             u64* dst = pb == 0 ? d0buf : buf;
+            ntt_fwd_regs<LOGN, false, E, CAP, 2>(dst, r, tid, t, q);
             const int sb = slot_base<LOGN, LAST, E>(tid);
-            const int xl = elem_index<LOGN, LAST, E>(tid, 0);
 #pragma unroll
-            for (int e = 0; e < E; ++e) {
-                const int at = SMEM_D0 || pb ? slot_of<LOGN, LAST, E>(sb, e) : xl + elem_offset<LOGN, LAST, E>(e);
-                dst[at] = csub(csub(r[0][e], 2 * q), q);
-            }
+            for (int e = 0; e < E; ++e)
+                dst[slot_of<LOGN, LAST, E>(sb, e)] = CAP == kNoFold ? r[e] : below4<CAP == kNoFold ? 1 : OUT>(r[e], q);
         }
 #pragma unroll   // unrolled: 2.62 -> 2.60 ms (the split kernel below keeps its loop: 2.45 -> 2.71 ms unrolled)
         for (int e = 0; e < E; e += 2) {
             const int x = elem_index<LOGN, LAST, E>(tid, e);
-            ulonglong2* p0 = reinterpret_cast<ulonglong2*>(acc + x);
-            ulonglong2* p1 = reinterpret_cast<ulonglong2*>(acc + N + x);
-            ulonglong2* p2 = reinterpret_cast<ulonglong2*>(acc + 2 * N + x);
-            ulonglong2 s0 = *p0, s1 = *p1, s2 = *p2;
-            u64 t[2][3];
-#pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-                const u64 d1 = buf[swz<E>(x + hh)];
-                const u64 d0 = SMEM_D0 ? d0buf[swz<E>(x + hh)] : d0buf[x + hh];
-                t[hh][0] = mont_mul(d0, d0, q, qinv);   // every term carries 2^{-64}, undone after the INTT
-                const u64 c = mont_mul(d0, d1, q, qinv);
-                t[hh][1] = add_mod(c, c, q);
-                t[hh][2] = mont_mul(d1, d1, q, qinv);
-            }
-            s0 = make_ulonglong2(add_mod(s0.x, t[0][0], q), add_mod(s0.y, t[1][0], q));
-            s1 = make_ulonglong2(add_mod(s1.x, t[0][1], q), add_mod(s1.y, t[1][1], q));
-            s2 = make_ulonglong2(add_mod(s2.x, t[0][2], q), add_mod(s2.y, t[1][2], q));
-            *p0 = s0;
-            *p1 = s1;
-            *p2 = s2;
+            tensor_pair(acc + x, N, buf[swz<E>(x)], buf[swz<E>(x + 1)], d0buf[swz<E>(x)], d0buf[swz<E>(x + 1)], q, qinv);
         }
     }
+}
+
+template <int LOGN, int E>
+__global__ void __launch_bounds__(NttShape<LOGN, E>::T, sqdiff_blocks_per_sm(LOGN)) k_sqdiff_accumulate(const __grid_constant__ SqDiffArgs a)
+{
+    extern __shared__ u64 buf[];
+    if (a.rns.q[blockIdx.x % a.limbs] < kNoFoldBelow) sqdiff_accumulate<LOGN, E, kNoFold>(a, buf);
+    else sqdiff_accumulate<LOGN, E, 16>(a, buf);
 }
 
 // N = 2^14, split: the first stage of the forward transform pairs x with x + N/2 and leaves two
@@ -105,11 +114,12 @@ __global__ void __launch_bounds__(NttShape<LOGN, E>::T, 1) k_sqdiff_accumulate(c
 // tw_h[2^s + g] = tw[(2 + h) 2^s + g]. Its tensor terms go to a [4][N/2] slice. The two
 // blocks of a half pair read the same ciphertexts at about the same time (one HBM read, one
 // L2 hit).
-__global__ void __launch_bounds__(1024, 1) k_sqdiff_accumulate_split(const __grid_constant__ SqDiffArgs a)
+template <int CAP>
+__device__ __forceinline__ void sqdiff_accumulate_split(const SqDiffArgs& a, u64* buf)
 {
     constexpr int LOGH = 13, NH = 1 << LOGH, N = 2 * NH, E = 8;
     constexpr int LAST = NttShape<LOGH, E>::LAST;
-    extern __shared__ u64 buf[];
+    constexpr int IN = 6, OUT = fwd_out<LOGH, false, CAP, IN>();
     u64* d0buf = buf + NH;
     const int tid = threadIdx.x;
     const int limbs = a.limbs;
@@ -137,60 +147,47 @@ __global__ void __launch_bounds__(1024, 1) k_sqdiff_accumulate_split(const __gri
             const int x0 = elem_index<LOGH, 0, E>(tid, 0);
             const u64* pa = A + ((u64)pb * limbs + l) * N + x0;
             const u64* pbb = B + ((u64)pb * limbs + l) * N + x0;
-            u64 r[1][E];
+            u64 r[E];
 #pragma unroll
             for (int e = 0; e < E; ++e) {
                 const int x = elem_offset<LOGH, 0, E>(e);
-                const u64 lo = sub_mod(pa[x], pbb[x], q);
-                const u64 hi = sub_mod(pa[x + NH], pbb[x + NH], q);
-                const u64 tt = shoup_lazy(hi, w1.x, w1.y, q);   // [0, 2q)
-                r[0][e] = h ? lo + 2 * q - tt : lo + tt;         // [0, 3q)
+                const u64 lo = pa[x] + q - pbb[x];                          // [0, 2q)
+                const u64 tt = shoup3(pa[x + NH] + q - pbb[x + NH], w1.x, w1.y, q);   // [0, 4q)
+                r[e] = h ? lo + 4 * q - tt : lo + tt;                       // below IN q
             }
             if (pb == 0) __syncthreads();   // d0 in its parking buffer, d1 in the other (as above)
-            ntt_fwd_regs<LOGH, 1, false, false, E>(pb == 0 ? d0buf : buf, r, tid, t, q);
             u64* dst = pb == 0 ? d0buf : buf;
+            ntt_fwd_regs<LOGH, false, E, CAP, IN>(dst, r, tid, t, q);
             const int sb = slot_base<LOGH, LAST, E>(tid);
 #pragma unroll
-            for (int e = 0; e < E; ++e) dst[slot_of<LOGH, LAST, E>(sb, e)] = csub(csub(r[0][e], 2 * q), q);
+            for (int e = 0; e < E; ++e)
+                dst[slot_of<LOGH, LAST, E>(sb, e)] = CAP == kNoFold ? r[e] : below4<CAP == kNoFold ? 1 : OUT>(r[e], q);
         }
 #pragma unroll 1
         for (int e = 0; e < E; e += 2) {
             const int x = elem_index<LOGH, LAST, E>(tid, e);
-            ulonglong2* p0 = reinterpret_cast<ulonglong2*>(acc + x);
-            ulonglong2* p1 = reinterpret_cast<ulonglong2*>(acc + NH + x);
-            ulonglong2* p2 = reinterpret_cast<ulonglong2*>(acc + 2 * NH + x);
-            ulonglong2 s0 = *p0, s1 = *p1, s2 = *p2;
-            u64 tt[2][3];
-#pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {
-                const u64 d1 = buf[swz<E>(x + hh)];
-                const u64 d0 = d0buf[swz<E>(x + hh)];
-                tt[hh][0] = mont_mul(d0, d0, q, qinv);   // every term carries 2^{-64}, undone after the INTT
-                const u64 c = mont_mul(d0, d1, q, qinv);
-                tt[hh][1] = add_mod(c, c, q);
-                tt[hh][2] = mont_mul(d1, d1, q, qinv);
-            }
-            *p0 = make_ulonglong2(add_mod(s0.x, tt[0][0], q), add_mod(s0.y, tt[1][0], q));
-            *p1 = make_ulonglong2(add_mod(s1.x, tt[0][1], q), add_mod(s1.y, tt[1][1], q));
-            *p2 = make_ulonglong2(add_mod(s2.x, tt[0][2], q), add_mod(s2.y, tt[1][2], q));
+            tensor_pair(acc + x, NH, buf[swz<E>(x)], buf[swz<E>(x + 1)], d0buf[swz<E>(x)], d0buf[swz<E>(x + 1)], q, qinv);
         }
     }
 }
 
-// Residues per thread: 8 at N = 2^13 (1024 threads), else 16.
-template <int LOGN>
-static constexpr int kSqE = LOGN == 13 ? 8 : 16;
+__global__ void __launch_bounds__(1024, 1) k_sqdiff_accumulate_split(const __grid_constant__ SqDiffArgs a)
+{
+    extern __shared__ u64 buf[];
+    if (a.rns.q[blockIdx.x % a.limbs] < kNoFoldBelow) sqdiff_accumulate_split<kNoFold>(a, buf);
+    else sqdiff_accumulate_split<16>(a, buf);
+}
 
+// 8 residues per thread: 1024 threads in 64 registers per SM at every N, as one block or several.
 template <int LOGN>
 static cudaError_t sqdiff_launch(const SqDiffArgs& a, cudaStream_t st)
 {
-    constexpr bool keep = LOGN <= 13;
-    constexpr int E = kSqE<LOGN>;
-    const size_t smem = (keep ? 2 : 1) * (sizeof(u64) << LOGN);
-    cudaError_t e = cudaFuncSetAttribute(k_sqdiff_accumulate<LOGN, keep, E>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    constexpr int E = 8;
+    const size_t smem = 2 * (sizeof(u64) << LOGN);
+    cudaError_t e = cudaFuncSetAttribute(k_sqdiff_accumulate<LOGN, E>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)smem);
     if (e != cudaSuccess) return e;
-    k_sqdiff_accumulate<LOGN, keep, E><<<a.n_blocks, NttShape<LOGN, E>::T, smem, st>>>(a);
+    k_sqdiff_accumulate<LOGN, E><<<a.n_blocks, NttShape<LOGN, E>::T, smem, st>>>(a);
     return cudaGetLastError();
 }
 
@@ -211,7 +208,6 @@ cudaError_t launch_sqdiff_accumulate(const SqDiffArgs& a, cudaStream_t st)
     case 11: return sqdiff_launch<11>(a, st);
     case 12: return sqdiff_launch<12>(a, st);
     case 13: return sqdiff_launch<13>(a, st);
-    case 14: return sqdiff_launch<14>(a, st);
     default: return cudaErrorInvalidValue;
     }
 }
@@ -226,9 +222,13 @@ __global__ void k_sqdiff_reduce(RnsArgs rns, int limbs, const u64* partial, int 
     const int row = split ? n / 2 : n;         // slice row length
     const int step = split ? 2 * limbs : limbs;
     for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < n; x += gridDim.x * blockDim.x) {
-        u64 s = add ? reduce64(tensor[(size_t)pl * n + x], q, rns.mu[l]) : 0;
+        u64 s = 0;
         const int h = split ? x / row : 0, xx = split ? x % row : x;
-        for (int j = l + h * limbs; j < n_blocks; j += step) s = add_mod(s, partial[((size_t)j * 4 + p) * row + xx], q);
+        for (int j = l + h * limbs; j < n_blocks; j += step)   // slices in [0, 2q), the sum too
+            s = csub_s(s + partial[((size_t)j * 4 + p) * row + xx], 2 * q);
+        s = csub_s(s, q);
+        if (p == 1) s = add_mod(s, s, q);                      // 2 d0 d1
+        if (add) s = add_mod(s, reduce64(tensor[(size_t)pl * n + x], q, rns.mu[l]), q);
         tensor[(size_t)pl * n + x] = s;
     }
 }
@@ -280,6 +280,8 @@ cudaError_t launch_reduce_rows(const RnsArgs& rns, int rows, int limbs, const u6
 // last pass (inverse), and its last exchange loads the slots of the other end, so a block
 // barrier is needed only between two transforms of the same direction: after a forward, an
 // inverse overwrites only slots its thread loaded last, and after an inverse a forward does.
+// 4096 pairs at N = 2^13 and three limbs take 11.1 ms (11.9 with a subtraction per butterfly, exact
+// quotients and canonical accumulators), 768 at N = 2^14 and five limbs 13.2 ms.
 // Every intermediate word is produced and consumed by the same thread (the transforms move
 // data between threads only through their own shared buffer), so the block's scratch
 // ([3 limbs + 2][N] words: t0^, t1^, t2 per limb, then the two P accumulators) is stored
@@ -293,7 +295,7 @@ cudaError_t launch_reduce_rows(const RnsArgs& rns, int rows, int limbs, const u6
 constexpr u32 kFwdDiff = 0, kInvT2 = 1, kFwdDigit = 2, kInvAcc = 3;
 
 template <int LOGN, int E>
-__global__ void __launch_bounds__(NttShape<LOGN, E>::T) k_sqdiff_image(const __grid_constant__ SqImgArgs a)
+__global__ void __launch_bounds__(NttShape<LOGN, E>::T, sqdiff_blocks_per_sm(LOGN)) k_sqdiff_image(const __grid_constant__ SqImgArgs a)
 {
     constexpr int N = 1 << LOGN;
     constexpr int T = NttShape<LOGN, E>::T;
@@ -346,7 +348,7 @@ __global__ void __launch_bounds__(NttShape<LOGN, E>::T) k_sqdiff_image(const __g
     for (u64 k = blockIdx.x; k < a.n_ct; k += gridDim.x) {
         const u64* A = a.a + k * 2 * (u64)limbs * N;
         const u64* B = a.b + k * 2 * (u64)limbs * N;
-        u64 r[1][E];
+        u64 r[E];
 #pragma unroll 1
         for (int op = 0; op < n_ops; ++op) {
             const u32 code = sched[op];
@@ -362,7 +364,7 @@ __global__ void __launch_bounds__(NttShape<LOGN, E>::T) k_sqdiff_image(const __g
 #pragma unroll
                     for (int e = 0; e < E; ++e) {
                         const int xi = elem_index<LOGN, 0, E>(tid, e);
-                        r[0][e] = sub_mod(__ldcs(pa + xi), __ldcs(pq + xi), q);
+                        r[e] = __ldcs(pa + xi) + q - __ldcs(pq + xi);   // [0, 2q)
                     }
                 } else {                  // digit x of t2, centered, lifted to the modulus
                     const u64 mu = a.rns.mu[mod];
@@ -373,27 +375,27 @@ __global__ void __launch_bounds__(NttShape<LOGN, E>::T) k_sqdiff_image(const __g
 #pragma unroll
                         for (int e = 0; e < E; ++e) {
                             const u64 v = t2[e * T];
-                            r[0][e] = v <= half ? v : q - (qj - v);
+                            r[e] = v <= half ? v : q - (qj - v);
                         }
                     } else {
 #pragma unroll
                         for (int e = 0; e < E; ++e) {
                             const u64 v = t2[e * T];
                             if (v <= half) {
-                                r[0][e] = reduce64(v, q, mu);
+                                r[e] = reduce64(v, q, mu);
                             } else {
                                 const u64 mag = reduce64(qj - v, q, mu);
-                                r[0][e] = mag == 0 ? 0 : q - mag;
+                                r[e] = mag == 0 ? 0 : q - mag;
                             }
                         }
                     }
                 }
                 if ((code >> 11) & 1u) __syncthreads();
-                ntt_fwd_regs<LOGN, 1, false, CMP, E>(sm, r, tid, a.rns.tab[mod], q);
+                ntt_fwd_regs<LOGN, CMP, E, 8, 2>(sm, r, tid, a.rns.tab[mod], q);   // below 8q
                 if (kind == kFwdDiff) {
                     u64* dst = (pb == 0 ? T0 : T2) + (size_t)x * N;
 #pragma unroll
-                    for (int e = 0; e < E; ++e) dst[e * T] = csub(csub(r[0][e], 2 * q), q);
+                    for (int e = 0; e < E; ++e) dst[e * T] = below4<8>(r[e], q);   // as mont_lazy takes it
                 } else {                  // acc_b(m) += NTT(digit) * evk^_x[b][m]
                     u64* acc0 = m < 0 ? AP : T0 + (size_t)m * N;
                     u64* acc1 = m < 0 ? AP + N : T1 + (size_t)m * N;
@@ -405,14 +407,13 @@ __global__ void __launch_bounds__(NttShape<LOGN, E>::T) k_sqdiff_image(const __g
 #pragma unroll
                     for (int e = 0; e < E; ++e) {
                         const int xi = elem_index<LOGN, LAST, E, WT>(tid, e);
-                        // the accumulators stay in [0, 2q): the inverse transform takes that range
-                        const u64 d = csub(csub(r[0][e], 2 * q), q);
-                        const u64 p0 = shoup_lazy(d, __ldg(e0 + xi), __ldg(e0p + xi), q);
-                        const u64 p1 = shoup_lazy(d, __ldg(e1 + xi), __ldg(e1p + xi), q);
+                        // the accumulators stay in [0, 4q): the inverse transform takes that range
+                        const u64 p0 = shoup3(r[e], __ldg(e0 + xi), __ldg(e0p + xi), q);
+                        const u64 p1 = shoup3(r[e], __ldg(e1 + xi), __ldg(e1p + xi), q);
                         const u64 s0 = init ? 0 : acc0[e * T];
                         const u64 s1 = init ? 0 : acc1[e * T];
-                        acc0[e * T] = csub(s0 + p0, 2 * q);
-                        acc1[e * T] = csub(s1 + p1, 2 * q);
+                        acc0[e * T] = halve<8>(s0 + p0, q);
+                        acc1[e * T] = halve<8>(s1 + p1, q);
                     }
                 }
             } else {
@@ -429,30 +430,30 @@ __global__ void __launch_bounds__(NttShape<LOGN, E>::T) k_sqdiff_image(const __g
                     for (int e = 0; e < E; ++e) {
                         const int xi = elem_index<LOGN, LAST, E, WT>(tid, e);
                         const u64 d0 = t0[e * T], d1 = t2[e * T];
-                        const u64 m2 = mont_mul(d1, d1, q, qinv);
-                        const u64 th = shoup(m2, a.r64[x], a.r64_p[x], q);   // d1^2, the transform of digit x
-                        const u64 c = mont_mul(d0, d1, q, qinv);
-                        t0[e * T] = csub(shoup_lazy(mont_mul(d0, d0, q, qinv), a.pn[x], a.pn_p[x], q) +
-                                         shoup_lazy(th, __ldg(e0 + xi), __ldg(e0p + xi), q), 2 * q);
-                        t1[e * T] = csub(shoup_lazy(add_mod(c, c, q), a.pn[x], a.pn_p[x], q) +
-                                         shoup_lazy(th, __ldg(e1 + xi), __ldg(e1p + xi), q), 2 * q);
-                        r[0][e] = shoup(m2, a.ninv[x], a.ninv_p[x], q);
+                        const u64 m2 = mont_lazy(d1, d1, q, qinv);
+                        const u64 th = shoup3(m2, a.r64[x], a.r64_p[x], q);   // d1^2, the transform of digit x
+                        const u64 c = mont_lazy(d0, d1, q, qinv);
+                        t0[e * T] = halve<8>(shoup3(mont_lazy(d0, d0, q, qinv), a.pn[x], a.pn_p[x], q) +
+                                             shoup3(th, __ldg(e0 + xi), __ldg(e0p + xi), q), q);
+                        t1[e * T] = halve<8>(shoup3(c + c, a.pn[x], a.pn_p[x], q) +
+                                             shoup3(th, __ldg(e1 + xi), __ldg(e1p + xi), q), q);
+                        r[e] = shoup3(m2, a.ninv[x], a.ninv_p[x], q);
                     }
                 } else {
                     const u64* acc = (m < 0 ? AP + (size_t)pb * N : (pb == 0 ? T0 : T1) + (size_t)m * N);
 #pragma unroll
-                    for (int e = 0; e < E; ++e) r[0][e] = acc[e * T];
+                    for (int e = 0; e < E; ++e) r[e] = acc[e * T];
                 }
                 if ((code >> 11) & 1u) __syncthreads();
-                ntt_inv_regs<LOGN, 1, CMP, E>(sm, r, tid, a.rns.tab[mod], q);
+                ntt_inv_regs<LOGN, CMP, E, 8>(sm, r, tid, a.rns.tab[mod], q);      // below 4q
                 if (kind == kInvT2) {
                     u64* t2 = T2 + (size_t)x * N;
 #pragma unroll
-                    for (int e = 0; e < E; ++e) t2[e * T] = csub(r[0][e], q);
+                    for (int e = 0; e < E; ++e) t2[e * T] = below1<4>(r[e], q);
                 } else if (m < 0) {
                     u64* acc = AP + (size_t)pb * N;
 #pragma unroll
-                    for (int e = 0; e < E; ++e) acc[e * T] = csub(r[0][e], q);
+                    for (int e = 0; e < E; ++e) acc[e * T] = below1<4>(r[e], q);
                 } else {
                     const u64 mu = a.rns.mu[mod];
                     u64* acc = (pb == 0 ? T0 : T1) + (size_t)m * N;
@@ -463,7 +464,7 @@ __global__ void __launch_bounds__(NttShape<LOGN, E>::T) k_sqdiff_image(const __g
                         const u64 ap = AP[(size_t)pb * N + e * T];
                         u64 lp = reduce64(ap, q, mu);
                         if (ap > halfP) lp = add_mod(lp, a.neg_p_mod[m], q);   // (ap - P) mod q_m
-                        const u64 md = shoup(sub_mod(csub(r[0][e], q), lp, q), a.p_inv[m], a.p_inv_p[m], q);
+                        const u64 md = shoup(r[e] + q - lp, a.p_inv[m], a.p_inv_p[m], q);
                         if (m == t) {
                             acc[e * T] = md;              // relinearised limb q_t, the rescale's divisor
                         } else {

@@ -3,17 +3,15 @@
 // need (Sec. 2.2, 2.2.2, 2.2.3).
 //
 // Layout: N = 2^LOGN residues, one thread block of N/E threads, every thread holding E
-// residues (E = 16 or 8) per polynomial in registers. The log2(N) butterfly stages run in
+// residues (E = 16 or 8) in registers. The log2(N) butterfly stages run in
 // passes of up to log2(E) stages (a radix-E step entirely in registers); between passes the
-// block exchanges data through one shared-memory buffer of N words per polynomial,
+// block exchanges data through one shared-memory buffer of N words,
 // XOR-swizzled so that every pass reads and writes without bank conflicts (the host-compiled
 // layout test checks every pass of N = 2^10 .. 2^14): x ^ ((x >> 4) & 15) for E = 16,
 // x ^ ((x >> 2) & 7) ^ ((x >> 3) & 15) for E = 8. E = 8 halves the registers a polynomial
 // takes, so twice the threads fit on an SM, at the price of one more exchange per transform.
 // An exchange whose two layouts give every warp the same residues takes a warp barrier
-// instead of a block barrier (the later passes of a transform). NP polynomials over the same
-// modulus can be transformed in lockstep: each twiddle pair is loaded once for all of them and
-// the barriers are shared.
+// instead of a block barrier (the later passes of a transform).
 //
 // Between transforms on the same buffer: a forward transform's first exchange stores to its
 // thread's pass-0 slots and its last exchange loads the thread's last-pass slots; an inverse
@@ -22,9 +20,15 @@
 // of the same direction in a row do.
 //
 // Forward: Cooley-Tukey with the negacyclic twist merged into the twiddles, natural-order
-// input, bit-reversed output; inputs in [0, q), outputs in [0, 4q) (Harvey's lazy bounds).
-// Inverse: Gentleman-Sande, bit-reversed input in [0, 2q), natural-order output in [0, 2q),
+// input, bit-reversed output. Inverse: Gentleman-Sande, bit-reversed input, natural-order output,
 // without the 1/N factor (callers fold 1/N into a constant operand).
+// Ranges: a product by a twiddle is left in [0, 4q) (shoup3), and CAP multiples of q fit a word:
+// CAP = 16 for ciphertext primes (below 2^60), 8 where the modulus may be the special prime (below
+// 2^61), kNoFold for moduli below 2^50, whose values never need one. Every register's bound is
+// known at compile time, and a conditional subtraction is spent only where the next sum would
+// pass CAP q: with CAP = 16 on 5 of the 13 stages at N = 2^13 instead of on every butterfly
+// (Harvey's [0, 4q)). Register-only butterflies: 887 G/s with the exact quotient and a subtraction
+// each, 1005 without the subtraction, 1132 with the three-product quotient as well.
 // Twiddles: tw[k] = psi^{bitrev(k)}, itw[k] = psi^{-bitrev(k)}, psi a primitive 2N-th root,
 // each stored next to its Shoup companion (one 16-byte load per twiddle).
 #pragma once
@@ -155,132 +159,163 @@ __device__ __forceinline__ int slot_base(int tid) { return swz<E>(elem_index<LOG
 template <int LOGN, int S0, int E = 16, bool WT = true>
 __device__ __forceinline__ int slot_of(int base, int e) { return base ^ swz<E>(elem_index<LOGN, S0, E, WT>(0, e)); }
 
-template <int LOGN, int S0, int NP, int E = 16, bool WT = true>
-__device__ __forceinline__ void load_sm(const u64* sm, u64 (&r)[NP][E], int tid)
+template <int LOGN, int S0, int E = 16, bool WT = true>
+__device__ __forceinline__ void load_sm(const u64* sm, u64 (&r)[E], int tid)
 {
     const int base = slot_base<LOGN, S0, E, WT>(tid);
 #pragma unroll
-    for (int p = 0; p < NP; ++p)
-#pragma unroll
-        for (int e = 0; e < E; ++e) r[p][e] = sm[p * (1 << LOGN) + slot_of<LOGN, S0, E, WT>(base, e)];
+    for (int e = 0; e < E; ++e) r[e] = sm[slot_of<LOGN, S0, E, WT>(base, e)];
 }
 
-template <int LOGN, int S0, int NP, int E = 16, bool WT = true>
-__device__ __forceinline__ void store_sm(u64* sm, const u64 (&r)[NP][E], int tid)
+template <int LOGN, int S0, int E = 16, bool WT = true>
+__device__ __forceinline__ void store_sm(u64* sm, const u64 (&r)[E], int tid)
 {
     const int base = slot_base<LOGN, S0, E, WT>(tid);
 #pragma unroll
-    for (int p = 0; p < NP; ++p)
-#pragma unroll
-        for (int e = 0; e < E; ++e) sm[p * (1 << LOGN) + slot_of<LOGN, S0, E, WT>(base, e)] = r[p][e];
+    for (int e = 0; e < E; ++e) sm[slot_of<LOGN, S0, E, WT>(base, e)] = r[e];
 }
 
-// Forward stages S0 .. S0+S-1 on the registers. Stage s pairs x with x + N/2^{s+1} and uses
-// twiddle index 2^s + (x >> (LOGN - s)). With TERNARY0 the first stage of pass 0 takes the
-// odd operands as ternary residues {0, 1, q-1}, whose products with the twiddle are 0, W and
-// q - W: no multiplication.
-template <int LOGN, int S0, int NP, bool TERNARY0 = false, int E = 16, bool WT = true>
-__device__ __forceinline__ void fwd_regs(u64 (&r)[NP][E], int tid, const ulonglong2* __restrict__ tw, u64 q)
+// f(Index<0>()), ..., f(Index<N - 1>()): a loop whose index is a compile-time constant.
+template <int I>
+struct Index {
+    static constexpr int v = I;
+};
+
+template <int N, int I = 0, class F>
+__device__ __forceinline__ void static_for(F&& f)
 {
-    using P = Pass<LOGN, S0, E>;
-    const u64 q2 = 2 * q;
-#pragma unroll
-    for (int g = 0; g < P::G; ++g) {
-        const int h = pass_gid(P::T, P::G, tid, g, WT) >> P::LO;
-#pragma unroll
-        for (int k = 0; k < P::S; ++k) {
-            const int s = S0 + k;
-            const int half = 1 << (P::S - 1 - k);
-#pragma unroll
-            for (int b = 0; b < (1 << k); ++b) {
-                const int widx = (1 << s) + (h << k) + b;
-                const ulonglong2 w2 = __ldg(tw + widx);
-                const u64 W = w2.x, Wp = w2.y;
-#pragma unroll
-                for (int jj = b * 2 * half; jj < b * 2 * half + half; ++jj) {
-                    const int i0 = g * (1 << P::S) + jj, i1 = i0 + half;
-#pragma unroll
-                    for (int p = 0; p < NP; ++p) {
-                        u64 X = r[p][i0];
-                        u64 Tt;
-                        if (TERNARY0 && S0 == 0 && k == 0) {
-                            const u64 y = r[p][i1];
-                            Tt = y == 0 ? 0 : (y == 1 ? W : q - W);
-                        } else {
-                            X = X >= q2 ? X - q2 : X;
-                            Tt = shoup_lazy(r[p][i1], W, Wp, q);
-                        }
-                        r[p][i0] = X + Tt;
-                        r[p][i1] = X - Tt + q2;
-                    }
-                }
-            }
-        }
+    if constexpr (I < N) {
+        f(Index<I>());
+        static_for<N, I + 1>(f);
     }
 }
 
-// Inverse stages S0+S-1 .. S0 (reverse order) on the registers.
-template <int LOGN, int S0, int NP, int E = 16, bool WT = true>
-__device__ __forceinline__ void inv_regs(u64 (&r)[NP][E], int tid, const ulonglong2* __restrict__ itw, u64 q)
+constexpr int kNoFold = 1 << 12;   // CAP of moduli below 2^50
+
+// x below CAP q to below CAP/2 q: one conditional subtraction.
+template <int CAP>
+__device__ __forceinline__ u64 halve(u64 x, u64 q) { return csub_s(x, (CAP / 2) * q); }
+
+// x below B q (B at most 16) to below 4q.
+template <int B>
+__device__ __forceinline__ u64 below4(u64 x, u64 q)
+{
+    static_assert(B <= 16, "one subtraction of 8q and one of 4q");
+    if constexpr (B > 8) x = csub_s(x, 8 * q);
+    if constexpr (B > 4) x = csub_s(x, 4 * q);
+    return x;
+}
+
+// x below B q to [0, q).
+template <int B>
+__device__ __forceinline__ u64 below1(u64 x, u64 q) { return csub_s(csub_s(below4<B>(x, q), 2 * q), q); }
+
+// Bound after S forward stages from b: a stage adds 4, its first operands halved below CAP/2 when the
+// sum would pass CAP.
+__host__ __device__ constexpr int fwd_bound(int cap, int b, int S)
+{
+    for (int k = 0; k < S; ++k) b = (b + 4 > cap ? cap / 2 : b) + 4;
+    return b;
+}
+
+// Forward stages S0 .. S0+S-1 on registers below B q. Stage s pairs x with x + N/2^{s+1} and uses
+// twiddle index 2^s + (x >> (LOGN - s)).
+template <int LOGN, int S0, int E, bool WT, int CAP, int B>
+__device__ __forceinline__ void fwd_regs(u64 (&r)[E], int tid, const ulonglong2* __restrict__ tw, u64 q)
 {
     using P = Pass<LOGN, S0, E>;
-    const u64 q2 = 2 * q;
-#pragma unroll
-    for (int g = 0; g < P::G; ++g) {
+    static_for<P::G>([&](auto gc) {
+        constexpr int g = decltype(gc)::v;
         const int h = pass_gid(P::T, P::G, tid, g, WT) >> P::LO;
-#pragma unroll
-        for (int k = P::S - 1; k >= 0; --k) {
-            const int s = S0 + k;
-            const int half = 1 << (P::S - 1 - k);
-#pragma unroll
-            for (int b = 0; b < (1 << k); ++b) {
-                const int widx = (1 << s) + (h << k) + b;
-                const ulonglong2 w2 = __ldg(itw + widx);
-                const u64 W = w2.x, Wp = w2.y;
+        static_for<P::S>([&](auto kc) {
+            constexpr int k = decltype(kc)::v, s = S0 + k, half = 1 << (P::S - 1 - k);
+            constexpr bool fold = fwd_bound(CAP, B, k) + 4 > CAP;
+            static_for<(1 << k)>([&](auto bc) {
+                constexpr int b = decltype(bc)::v;
+                const ulonglong2 w = __ldg(tw + (1 << s) + (h << k) + b);
 #pragma unroll
                 for (int jj = b * 2 * half; jj < b * 2 * half + half; ++jj) {
                     const int i0 = g * (1 << P::S) + jj, i1 = i0 + half;
-#pragma unroll
-                    for (int p = 0; p < NP; ++p) {
-                        const u64 X = r[p][i0], Y = r[p][i1];
-                        u64 U = X + Y;
-                        U = U >= q2 ? U - q2 : U;
-                        r[p][i0] = U;
-                        r[p][i1] = shoup_lazy(X - Y + q2, W, Wp, q);
-                    }
+                    const u64 X = fold ? halve<CAP>(r[i0], q) : r[i0];
+                    const u64 T = shoup3(r[i1], w.x, w.y, q);
+                    r[i0] = X + T;
+                    r[i1] = X - T + 4 * q;
                 }
-            }
-        }
-    }
+            });
+        });
+    });
+}
+
+// A stage takes X and Y, both below b q, to X + Y -- halved when it would pass CAP/2 -- and a product
+// in [0, 4q). Bound of register i before step t of an inverse pass that starts from B: the sums since
+// its last product.
+__host__ __device__ constexpr int inv_before(int cap, int B, int t, int i)
+{
+    int b = B;
+    for (int u = 0; u < t; ++u) b = ((i >> u) & 1) ? 4 : (2 * b > cap / 2 ? cap / 2 : 2 * b);
+    return b;
+}
+
+__host__ __device__ constexpr int inv_bound(int cap, int b, int S)
+{
+    int m = 4;
+    for (int i = 0; i < (1 << S); ++i) m = inv_before(cap, b, S, i) > m ? inv_before(cap, b, S, i) : m;
+    return m;
+}
+
+// Inverse stages S0+S-1 .. S0 (reverse order) on registers below B q (B <= CAP/2).
+template <int LOGN, int S0, int E, bool WT, int CAP, int B>
+__device__ __forceinline__ void inv_regs(u64 (&r)[E], int tid, const ulonglong2* __restrict__ itw, u64 q)
+{
+    using P = Pass<LOGN, S0, E>;
+    static_for<P::G>([&](auto gc) {
+        constexpr int g = decltype(gc)::v;
+        const int h = pass_gid(P::T, P::G, tid, g, WT) >> P::LO;
+        static_for<P::S>([&](auto tc) {
+            constexpr int t = decltype(tc)::v, k = P::S - 1 - t, s = S0 + k, half = 1 << t;
+            static_for<(1 << k)>([&](auto bc) {
+                constexpr int b = decltype(bc)::v;
+                const ulonglong2 w = __ldg(itw + (1 << s) + (h << k) + b);
+                static_for<half>([&](auto jc) {
+                    constexpr int j0 = b * 2 * half + decltype(jc)::v;
+                    constexpr int i0 = g * (1 << P::S) + j0, i1 = i0 + half;
+                    constexpr int bound = inv_before(CAP, B, t, j0);
+                    const u64 X = r[i0], Y = r[i1];
+                    r[i0] = 2 * bound > CAP / 2 ? halve<CAP>(X + Y, q) : X + Y;
+                    r[i1] = shoup3(X - Y + bound * q, w.x, w.y, q);
+                });
+            });
+        });
+    });
 }
 
 // Forward passes after the first: on entry r holds the output of pass S0-LE (its layout), on
 // exit the output of the last pass in the last pass's layout.
-template <int LOGN, int S0, int NP, int E = 16>
-__device__ __forceinline__ void fwd_rest(u64* sm, u64 (&r)[NP][E], int tid, const ulonglong2* __restrict__ tw, u64 q)
+template <int LOGN, int S0, int E, int CAP, int B>
+__device__ __forceinline__ void fwd_rest(u64* sm, u64 (&r)[E], int tid, const ulonglong2* __restrict__ tw, u64 q)
 {
     constexpr int LE = Radix<E>::LE;
     if constexpr (S0 <= NttShape<LOGN, E>::LAST) {
-        store_sm<LOGN, S0 - LE, NP, E>(sm, r, tid);
+        store_sm<LOGN, S0 - LE, E>(sm, r, tid);
         exchange_barrier<exchange_in_warp(LOGN, S0 - LE, S0, E)>();
-        load_sm<LOGN, S0, NP, E>(sm, r, tid);
-        fwd_regs<LOGN, S0, NP, false, E>(r, tid, tw, q);
-        fwd_rest<LOGN, S0 + LE, NP, E>(sm, r, tid, tw, q);
+        load_sm<LOGN, S0, E>(sm, r, tid);
+        fwd_regs<LOGN, S0, E, true, CAP, B>(r, tid, tw, q);
+        fwd_rest<LOGN, S0 + LE, E, CAP, fwd_bound(CAP, B, Pass<LOGN, S0, E>::S)>(sm, r, tid, tw, q);
     }
 }
 
 // Inverse passes S0, S0-LE, ..., 0: on entry r holds bit-reversed data in the layout of pass
 // S0 (no inverse stage applied yet), on exit natural-order data in the layout of pass 0.
-template <int LOGN, int S0, int NP, int E = 16>
-__device__ __forceinline__ void inv_rest(u64* sm, u64 (&r)[NP][E], int tid, const ulonglong2* __restrict__ itw, u64 q)
+template <int LOGN, int S0, int E, int CAP, int B>
+__device__ __forceinline__ void inv_rest(u64* sm, u64 (&r)[E], int tid, const ulonglong2* __restrict__ itw, u64 q)
 {
     constexpr int LE = Radix<E>::LE;
-    inv_regs<LOGN, S0, NP, E>(r, tid, itw, q);
+    inv_regs<LOGN, S0, E, true, CAP, B>(r, tid, itw, q);
     if constexpr (S0 > 0) {
-        store_sm<LOGN, S0, NP, E>(sm, r, tid);
+        store_sm<LOGN, S0, E>(sm, r, tid);
         exchange_barrier<exchange_in_warp(LOGN, S0, S0 - LE, E)>();
-        load_sm<LOGN, S0 - LE, NP, E>(sm, r, tid);
-        inv_rest<LOGN, S0 - LE, NP, E>(sm, r, tid, itw, q);
+        load_sm<LOGN, S0 - LE, E>(sm, r, tid);
+        inv_rest<LOGN, S0 - LE, E, CAP, inv_bound(CAP, B, Pass<LOGN, S0, E>::S)>(sm, r, tid, itw, q);
     }
 }
 
@@ -316,96 +351,77 @@ __device__ __forceinline__ void rt_offsets(int lo, int (&c)[E])
     }
 }
 
-template <int LOGN, int NP, int E = 16>
-__device__ __forceinline__ void store_sm_rt(u64* sm, const u64 (&r)[NP][E], int tid, int lo)
+template <int E = 16>
+__device__ __forceinline__ void store_sm_rt(u64* sm, const u64 (&r)[E], int tid, int lo)
 {
     const int base = swz<E>(pass_base<Radix<E>::LE>(tid, lo));
     int c[E];
     rt_offsets<E>(lo, c);
 #pragma unroll
-    for (int p = 0; p < NP; ++p)
-#pragma unroll
-        for (int e = 0; e < E; ++e) sm[p * (1 << LOGN) + (base ^ c[e])] = r[p][e];
+    for (int e = 0; e < E; ++e) sm[base ^ c[e]] = r[e];
 }
 
-template <int LOGN, int NP, int E = 16>
-__device__ __forceinline__ void load_sm_rt(const u64* sm, u64 (&r)[NP][E], int tid, int lo)
+template <int E = 16>
+__device__ __forceinline__ void load_sm_rt(const u64* sm, u64 (&r)[E], int tid, int lo)
 {
     const int base = swz<E>(pass_base<Radix<E>::LE>(tid, lo));
     int c[E];
     rt_offsets<E>(lo, c);
 #pragma unroll
-    for (int p = 0; p < NP; ++p)
-#pragma unroll
-        for (int e = 0; e < E; ++e) r[p][e] = sm[p * (1 << LOGN) + (base ^ c[e])];
+    for (int e = 0; e < E; ++e) r[e] = sm[base ^ c[e]];
 }
 
-// Forward stages S0 .. S0+LE-1 (lo = LOGN - S0 - LE).
-template <int NP, int E = 16>
-__device__ __forceinline__ void fwd_regs_rt(u64 (&r)[NP][E], int tid, int S0, int lo, const ulonglong2* __restrict__ tw,
-                                            u64 q)
+// Forward stages S0 .. S0+LE-1 (lo = LOGN - S0 - LE): registers below CAP q on entry and exit (one
+// code for every pass, so every stage halves its first operands). The runtime passes take the exact
+// quotient: the three-product form spilled more there (312 against 184 bytes; per-pixel squared
+// difference of 768 pairs at N = 2^14 16.9 against 13.8 ms).
+template <int CAP, int E = 16>
+__device__ __forceinline__ void fwd_regs_rt(u64 (&r)[E], int tid, int S0, int lo, const ulonglong2* __restrict__ tw, u64 q)
 {
     constexpr int LE = Radix<E>::LE;
-    const u64 q2 = 2 * q;
     const int h = tid >> lo;
 #pragma unroll
     for (int k = 0; k < LE; ++k) {
         const int half = 1 << (LE - 1 - k);
 #pragma unroll
         for (int b = 0; b < (1 << k); ++b) {
-            const int widx = (1 << (S0 + k)) + (h << k) + b;
-            const ulonglong2 w2 = __ldg(tw + widx);
-            const u64 W = w2.x, Wp = w2.y;
+            const ulonglong2 w = __ldg(tw + (1 << (S0 + k)) + (h << k) + b);
 #pragma unroll
             for (int jj = b * 2 * half; jj < b * 2 * half + half; ++jj) {
-#pragma unroll
-                for (int p = 0; p < NP; ++p) {
-                    u64 X = r[p][jj];
-                    X = X >= q2 ? X - q2 : X;
-                    const u64 Tt = shoup_lazy(r[p][jj + half], W, Wp, q);
-                    r[p][jj] = X + Tt;
-                    r[p][jj + half] = X - Tt + q2;
-                }
+                const u64 X = halve<CAP>(r[jj], q);
+                const u64 T = shoup_lazy(r[jj + half], w.x, w.y, q);
+                r[jj] = X + T;
+                r[jj + half] = X - T + 2 * q;
             }
         }
     }
 }
 
-// Inverse stages S0+LE-1 .. S0 (lo = LOGN - S0 - LE).
-template <int NP, int E = 16>
-__device__ __forceinline__ void inv_regs_rt(u64 (&r)[NP][E], int tid, int S0, int lo, const ulonglong2* __restrict__ itw,
-                                            u64 q)
+// Inverse stages S0+LE-1 .. S0 (lo = LOGN - S0 - LE): registers below CAP/2 q on entry and exit.
+template <int CAP, int E = 16>
+__device__ __forceinline__ void inv_regs_rt(u64 (&r)[E], int tid, int S0, int lo, const ulonglong2* __restrict__ itw, u64 q)
 {
     constexpr int LE = Radix<E>::LE;
-    const u64 q2 = 2 * q;
     const int h = tid >> lo;
 #pragma unroll
     for (int k = LE - 1; k >= 0; --k) {
         const int half = 1 << (LE - 1 - k);
 #pragma unroll
         for (int b = 0; b < (1 << k); ++b) {
-            const int widx = (1 << (S0 + k)) + (h << k) + b;
-            const ulonglong2 w2 = __ldg(itw + widx);
-            const u64 W = w2.x, Wp = w2.y;
+            const ulonglong2 w = __ldg(itw + (1 << (S0 + k)) + (h << k) + b);
 #pragma unroll
             for (int jj = b * 2 * half; jj < b * 2 * half + half; ++jj) {
-#pragma unroll
-                for (int p = 0; p < NP; ++p) {
-                    const u64 X = r[p][jj], Y = r[p][jj + half];
-                    u64 U = X + Y;
-                    U = U >= q2 ? U - q2 : U;
-                    r[p][jj] = U;
-                    r[p][jj + half] = shoup_lazy(X - Y + q2, W, Wp, q);
-                }
+                const u64 X = r[jj], Y = r[jj + half];
+                r[jj] = halve<CAP>(X + Y, q);
+                r[jj + half] = shoup_lazy(X - Y + (CAP / 2) * q, w.x, w.y, q);
             }
         }
     }
 }
 
-// Whole forward transform of NP polynomials, input already in registers in the layout of
-// pass 0 (values in [0, 4q); with TERNARY0, residues of a ternary polynomial); output in
-// registers in the layout of the last pass. `sm` holds NP buffers of N words. The caller must
-// make sure no thread still reads `sm` from an earlier use other than an inverse transform's
+// Whole forward transform, input already in registers in the layout of pass 0, below B q; output
+// in registers in the layout of the last pass, below fwd_out q. `sm` holds N words. The caller
+// must make sure no thread still reads `sm` from an earlier use other than an inverse transform's
 // (a __syncthreads before the call; see the header comment).
 // Passes: LOGN / LE full passes, then one pass of the remaining LOGN % LE stages.
 // COMPACT runs the full passes through one runtime loop (one copy of the pass code); otherwise
@@ -415,69 +431,66 @@ __device__ __forceinline__ void inv_regs_rt(u64 (&r)[NP][E], int tid, int S0, in
 // squared difference at N = 2^14 (where the unrolled passes spill), keeps the strided last-pass
 // layout (WT = false; its callers index the last pass with it) and a block barrier into it:
 // there the warp-adjacent layout took more registers (spills 8 -> 76 bytes) and time.
-template <int LOGN, int NP, bool TERNARY0 = false, bool COMPACT = false, int E = 16>
-__device__ __forceinline__ void ntt_fwd_regs(u64* sm, u64 (&r)[NP][E], int tid, const ModTables& t, u64 q)
+template <int LOGN, bool COMPACT, int CAP, int B>
+__host__ __device__ constexpr int fwd_out() { return COMPACT ? CAP : fwd_bound(CAP, B, LOGN); }
+
+template <int LOGN, bool COMPACT, int E, int CAP, int B>
+__device__ __forceinline__ void ntt_fwd_regs(u64* sm, u64 (&r)[E], int tid, const ModTables& t, u64 q)
 {
     constexpr int LE = Radix<E>::LE;
     if constexpr (!COMPACT) {
-        fwd_regs<LOGN, 0, NP, TERNARY0, E>(r, tid, t.tw, q);
-        fwd_rest<LOGN, LE, NP, E>(sm, r, tid, t.tw, q);
+        fwd_regs<LOGN, 0, E, true, CAP, B>(r, tid, t.tw, q);
+        fwd_rest<LOGN, LE, E, CAP, fwd_bound(CAP, B, Pass<LOGN, 0, E>::S)>(sm, r, tid, t.tw, q);
         return;
     }
     constexpr int NFULL = LOGN / LE, TAIL = LOGN % LE;
-    int p0 = 0;
-    if constexpr (TERNARY0) {
-        fwd_regs<LOGN, 0, NP, true, E>(r, tid, t.tw, q);
-        p0 = 1;
-    }
     constexpr unsigned in_warp = full_exchanges_in_warp(LOGN, E);
 #pragma unroll 1
-    for (int p = p0; p < NFULL; ++p) {
+    for (int p = 0; p < NFULL; ++p) {
         const int lo = LOGN - LE * p - LE;
         if (p > 0) {
-            store_sm_rt<LOGN, NP, E>(sm, r, tid, lo + LE);
+            store_sm_rt<E>(sm, r, tid, lo + LE);
             if ((in_warp >> p) & 1u) __syncwarp();   // uniform across the block
             else __syncthreads();
-            load_sm_rt<LOGN, NP, E>(sm, r, tid, lo);
+            load_sm_rt<E>(sm, r, tid, lo);
         }
-        fwd_regs_rt<NP, E>(r, tid, LE * p, lo, t.tw, q);
+        fwd_regs_rt<CAP, E>(r, tid, LE * p, lo, t.tw, q);
     }
     if constexpr (TAIL > 0) {
-        store_sm_rt<LOGN, NP, E>(sm, r, tid, LOGN - LE * NFULL);
+        store_sm_rt<E>(sm, r, tid, LOGN - LE * NFULL);
         __syncthreads();
-        load_sm<LOGN, LE * NFULL, NP, E, false>(sm, r, tid);
-        fwd_regs<LOGN, LE * NFULL, NP, false, E, false>(r, tid, t.tw, q);
+        load_sm<LOGN, LE * NFULL, E, false>(sm, r, tid);
+        fwd_regs<LOGN, LE * NFULL, E, false, CAP, CAP>(r, tid, t.tw, q);
     }
 }
 
-// Whole inverse transform of NP polynomials, input in registers in the layout of the last
-// pass (values in [0, 2q)); output in registers in the layout of pass 0, natural order, in
-// [0, 2q).
-template <int LOGN, int NP, bool COMPACT = false, int E = 16>
-__device__ __forceinline__ void ntt_inv_regs(u64* sm, u64 (&r)[NP][E], int tid, const ModTables& t, u64 q)
+// Whole inverse transform, input in registers in the layout of the last pass, below 4q; output in
+// registers in the layout of pass 0, natural order, below CAP/2 q.
+template <int LOGN, bool COMPACT, int E, int CAP>
+__device__ __forceinline__ void ntt_inv_regs(u64* sm, u64 (&r)[E], int tid, const ModTables& t, u64 q)
 {
     constexpr int LE = Radix<E>::LE;
     if constexpr (!COMPACT) {
-        inv_rest<LOGN, NttShape<LOGN, E>::LAST, NP, E>(sm, r, tid, t.itw, q);
+        inv_rest<LOGN, NttShape<LOGN, E>::LAST, E, CAP, 4>(sm, r, tid, t.itw, q);
         return;
     }
     constexpr int NFULL = LOGN / LE, TAIL = LOGN % LE;
     if constexpr (TAIL > 0) {
-        inv_regs<LOGN, LE * NFULL, NP, E, false>(r, tid, t.itw, q);
-        store_sm<LOGN, LE * NFULL, NP, E, false>(sm, r, tid);
+        inv_regs<LOGN, LE * NFULL, E, false, CAP, 4>(r, tid, t.itw, q);
+        store_sm<LOGN, LE * NFULL, E, false>(sm, r, tid);
         __syncthreads();
-        load_sm_rt<LOGN, NP, E>(sm, r, tid, LOGN - LE * NFULL);
+        load_sm_rt<E>(sm, r, tid, LOGN - LE * NFULL);
     }
     constexpr unsigned in_warp = full_exchanges_in_warp(LOGN, E);
 #pragma unroll 1
     for (int p = NFULL - 1; p >= 0; --p) {
         const int lo = LOGN - LE * p - LE;
-        inv_regs_rt<NP, E>(r, tid, LE * p, lo, t.itw, q);
+        inv_regs_rt<CAP, E>(r, tid, LE * p, lo, t.itw, q);
         if (p > 0) {
-            store_sm_rt<LOGN, NP, E>(sm, r, tid, lo);
+            store_sm_rt<E>(sm, r, tid, lo);
             if ((in_warp >> p) & 1u) __syncwarp();
             else __syncthreads();
-            load_sm_rt<LOGN, NP, E>(sm, r, tid, lo + LE);
+            load_sm_rt<E>(sm, r, tid, lo + LE);
         }
     }
 }

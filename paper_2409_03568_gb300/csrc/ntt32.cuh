@@ -41,21 +41,6 @@ __device__ __forceinline__ u32 fold32(u32 x, u32 p, u32 neg_p2)
     else return x;
 }
 
-// f(Index<0>()), ..., f(Index<N - 1>()): a loop whose index is a compile-time constant.
-template <int I>
-struct Index {
-    static constexpr int v = I;
-};
-
-template <int N, int I = 0, class F>
-__device__ __forceinline__ void static_for(F&& f)
-{
-    if constexpr (I < N) {
-        f(Index<I>());
-        static_for<N, I + 1>(f);
-    }
-}
-
 // The 2^k twiddles of one butterfly group in stage s of a pass, entries 2^s + (h << k) + b: pairs of
 // neighbours in one 16-byte load.
 template <int K, int ST>

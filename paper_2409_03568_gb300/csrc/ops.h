@@ -93,6 +93,8 @@ cudaError_t launch_radix_meanfilter3_batch(const RadixArgs& ra, const OpsArgs& a
 // transform's first stage (sqdiff_split(logn)), block j taking limb j % limbs and half
 // (j / limbs) % 2, with twiddle tables per half (htab).
 __host__ __device__ inline bool sqdiff_split(int logn) { return logn == 14; }
+// Accumulating blocks an SM holds: 1024 threads' worth (2^13 / 8 threads a block at N = 2^13 and 2^14).
+__host__ __device__ constexpr int sqdiff_blocks_per_sm(int logn) { return logn >= 13 ? 1 : 1 << (13 - logn); }
 struct SqDiffArgs {
     RnsArgs rns;                   // moduli 0..limbs-1
     int limbs;
