@@ -120,12 +120,13 @@ ichee_status meanfilter_chunked(ichee_ctx* c, const uint64_t* const* a, const ic
     set_rescale(c, base);
     fold_constants(c, base);
     ls.threads = mf_batch_threads(base.limbs, ls.threads, c->mf_staged != 0);
-    const int chunks = (c->n / 2) / ls.threads;
     for (uint32_t first = 0; first < n; first += kMaxSegs) {
         const int cnt = (int)std::min<uint32_t>(kMaxSegs, n - first);
         SegTable t;
         std::memset(&t, 0, sizeof(t));
-        fill_starts(t, first, cnt, [&](uint32_t i) { return (u64)ma[i].h * chunks * 2 * ma[i].c; });
+        fill_starts(t, first, cnt, [&](uint32_t i) {
+            return mf_items(c->logn, base.limbs, ls.threads, c->mf_staged != 0, ma[i].h, ma[i].c);
+        });
         for (int s = 0; s < cnt; ++s) {
             const uint32_t i = first + s;
             t.in0[s] = a[i];

@@ -103,23 +103,28 @@ struct LookupArgs {
 // belongs to segment s with start[s] <= g < start[s + 1] and is item g - start[s] of it. The
 // table travels as a kernel argument (no device memory, nothing to allocate).
 constexpr int kMaxSegs = 64;
-struct SegTable {
+template <int SEGS>
+struct SegTableOf {
     int n;
-    u64 start[kMaxSegs + 1];
-    const uint8_t* px[kMaxSegs];      // pixel input (encryption)
-    const u64* in0[kMaxSegs];         // ciphertext inputs
-    const u64* in1[kMaxSegs];
-    u64* out[kMaxSegs];               // ciphertext output
-    u64* out2[kMaxSegs];              // second ciphertext output (fused encrypt + filter)
-    double* dout[kMaxSegs];           // decoded output (decryption)
-    u64 seed[kMaxSegs];
-    uint32_t h[kMaxSegs], w[kMaxSegs], c[kMaxSegs], c1[kMaxSegs];
+    u64 start[SEGS + 1];
+    const uint8_t* px[SEGS];      // pixel input (encryption)
+    const u64* in0[SEGS];         // ciphertext inputs
+    const u64* in1[SEGS];
+    u64* out[SEGS];               // ciphertext output
+    u64* out2[SEGS];              // second ciphertext output (fused encrypt + filter)
+    double* dout[SEGS];           // decoded output (decryption)
+    u64 seed[SEGS];
+    uint32_t h[SEGS], w[SEGS], c[SEGS], c1[SEGS];
     // mean filter of a band: output rows y0 .. y0 + rows - 1 (rows = 0: the whole image), the
     // input holding the image's rows from row0 on
-    uint32_t y0[kMaxSegs], rows[kMaxSegs], row0[kMaxSegs];
-    double scale[kMaxSegs];
-    u64 kadd[kMaxSegs][kMaxPrimes];   // per-segment plaintext constant residues
+    uint32_t y0[SEGS], rows[SEGS], row0[SEGS];
+    double scale[SEGS];
+    u64 kadd[SEGS][kMaxPrimes];   // per-segment plaintext constant residues
 };
+typedef SegTableOf<kMaxSegs> SegTable;
+typedef SegTableOf<1> OneSeg;     // a single image: a hundredth of the arguments to pass
+
+__device__ __forceinline__ int seg_of(const OneSeg&, u64) { return 0; }
 
 __device__ __forceinline__ int seg_of(const SegTable& t, u64 g)
 {

@@ -44,8 +44,8 @@ struct RescaleQuot {
 __device__ __forceinline__ RescaleQuot rescale_quot(u64 st, const OpsArgs& a, int t)
 {
     const u64 q = a.q[t];
-    st = st >= 8 * q ? st - 8 * q : st;
-    st = st >= 4 * q ? st - 4 * q : st;
+    st = csub_s(st, 8 * q);
+    st = csub_s(st, 4 * q);
     u64 hi = mulhi(st, a.k0p[t]);
     u64 r = st * a.k0[t] - hi * q;   // in [0, 2q): K S' = hi q + r
     if (r >= q) { r -= q; hi += 1; }
@@ -58,8 +58,7 @@ __device__ __forceinline__ u64 rescale_quot_limb(u64 sj, const RescaleQuot& rq, 
 {
     const u64 qj = a.q[j];
     u64 v = shoup_lazy(sj + a.mq[j] - rq.s, a.k0r[j], a.k0rp[j], qj) + rq.u;   // in [0, 3 q_j)
-    v = v >= 2 * qj ? v - 2 * qj : v;
-    return v >= qj ? v - qj : v;
+    return csub_s(csub_s(v, 2 * qj), qj);
 }
 
 // Elementwise add / sub of two images with the same shape (Sec. 2.2.3, Sec. 3.3).
@@ -188,58 +187,101 @@ __device__ __forceinline__ void mf_store(const OpsArgs& a, const ulonglong2 (&cl
     }
 }
 
-// Fused 3x3 mean filter (Sec. 4.4.1; borders clamp to the edge): out(y,x) = Rescale(K9 * sum of the 9
-// clamp-to-edge neighbours). One block per (row y, channel, poly, coefficient chunk); each
-// thread owns one coefficient pair and walks the row left to right keeping the three column
-// sums of the window in registers, so every input row is loaded once per output row. Residues
-// are below 2^60, so the 9-term sums fit 64 bits unreduced and go straight into the Shoup
-// products (K9 for the dropped limb, K9 q_t^{-1} for the kept ones).
-// in0 holds the image's rows from row0 on, out0 its output rows from yout0 on (0 and 0 for a
-// whole image); h is the height of the whole image (the clamping rows).
+// One output coefficient from the unreduced 9-term sums of its limbs, stored to o[j * n] per kept
+// limb: fused multiply by K9 and rescale.
 template <int LIMBS>
-__device__ __forceinline__ void meanfilter_row(const OpsArgs& a, const u64* in0, u64* out0, int h, int w, int C, int y,
-                                               int chunk, int b, int ch, int row0 = 0, int yout0 = 0)
+__device__ __forceinline__ void mf_store1(const OpsArgs& a, const u64 (&s)[LIMBS], u64* o, int n)
 {
-    const int n = 1 << a.logn;
-    const int c2 = chunk * blockDim.x + threadIdx.x;  // coefficient-pair index
-    const u64 ct_len2 = (u64)2 * LIMBS * (n / 2);
-    const u64 out_len2 = (u64)2 * (LIMBS - 1) * (n / 2);
-    const ulonglong2* in = reinterpret_cast<const ulonglong2*>(in0) + (u64)b * LIMBS * (n / 2) + c2;
-    ulonglong2* out = reinterpret_cast<ulonglong2*>(out0) + (u64)b * (LIMBS - 1) * (n / 2) + c2;
-    const int ym = y > 0 ? y - 1 : 0, yp = y + 1 < h ? y + 1 : h - 1;
-    const int half = n / 2;
-    // the three input rows at column 0 and the output row at column 0; one column further is a
-    // fixed stride of C ciphertexts (pointer adds, no per-column 64-bit products)
-    const ulonglong2* r0 = in + ((u64)(ym - row0) * w * C + ch) * ct_len2;
-    const ulonglong2* r1 = in + ((u64)(y - row0) * w * C + ch) * ct_len2;
-    const ulonglong2* r2 = in + ((u64)(yp - row0) * w * C + ch) * ct_len2;
-    const u64 in_step = (u64)C * ct_len2;
-    ulonglong2* o = out + ((u64)(y - yout0) * w * C + ch) * out_len2;
-    const u64 out_step = (u64)C * out_len2;
+    if (a.k0_same) {
+        const RescaleQuot rq = rescale_quot(s[LIMBS - 1], a, LIMBS - 1);
+#pragma unroll
+        for (int j = 0; j < LIMBS - 1; ++j) __stcs(o + j * n, rescale_quot_limb(s[j], rq, j, a));
+    } else {
+        const u64 t = shoup(s[LIMBS - 1], a.k0[LIMBS - 1], a.k0p[LIMBS - 1], a.q[LIMBS - 1]);
+#pragma unroll
+        for (int j = 0; j < LIMBS - 1; ++j)
+            __stcs(o + j * n, rescale_fold(shoup_lazy(s[j], a.k0r[j], a.k0rp[j], a.q[j]), t, j, a));
+    }
+}
 
-    ulonglong2 col[3][LIMBS];
-    auto column = [&](int xx, ulonglong2 (&dst)[LIMBS]) {
-        const u64 off = (u64)xx * in_step;
+// Fused 3x3 mean filter (Sec. 4.4.1; borders clamp to the edge): out(y,x) = Rescale(K9 * sum of the 9
+// clamp-to-edge neighbours). One block per (group of R rows from y, channel, poly, coefficient
+// chunk); each thread owns one coefficient and walks the R rows left to right, so a column's R + 2
+// residues per limb are loaded once for its R outputs: each input row is read (R + 2) / R times
+// instead of three, through an L2 that else delivers more bytes than HBM does. Of the column sums
+// (three rows, unreduced) it keeps the last one and the sum of the last two. Residues are below
+// 2^60, so the 9-term sums fit 64 bits and go straight into the Shoup products (K9 for the dropped
+// limb, K9 q_t^{-1} for the kept ones).
+// in0 holds the image's rows from row0 on, out0 its output rows from yout0 on (0 and 0 for a
+// whole image); h is the height of the whole image (the clamping rows), y_end the end of the output
+// rows.
+// The next column's residues are loaded before the current column's outputs are computed: with R
+// small enough that nothing spills (128 registers, 512 threads per SM) the loads in flight cover
+// the memory latency. Measured (one 16-byte pair of coefficients and one row per thread before):
+// 128x128x3 at N = 2^13, four limbs 8.66 -> 6.98 ms (6.5 TB/s of input read once and output, 0.95 of
+// copy bandwidth); 128x128, three limbs 1.98 -> 1.77 ms; 48x48x3 at N = 2^14, five limbs 2.98 -> 2.60
+// ms. Without the early loads R = 2 took 10.3 ms at four limbs; R = 4 there and R = 5 at three limbs
+// spill (8.6 and 2.0 ms), R = 1 at four limbs takes 9.4.
+template <int LIMBS>
+static constexpr int kMfRows = LIMBS == 3 ? 4 : LIMBS <= 4 ? 3 : LIMBS <= 6 ? 2 : 1;
+
+template <int LIMBS>
+__device__ __forceinline__ void meanfilter_rows(const OpsArgs& a, const u64* in0, u64* out0, int h, int w, int C, int y,
+                                                int y_end, int chunk, int b, int ch, int row0, int yout0)
+{
+    constexpr int R = kMfRows<LIMBS>;
+    const int n = 1 << a.logn;
+    const int c = chunk * blockDim.x + threadIdx.x;   // coefficient
+    const u64 in_step = (u64)C * 2 * LIMBS * n, out_step = (u64)C * 2 * (LIMBS - 1) * n;   // one column further
+    const u64* src[R + 2];   // the input rows y - 1 .. y + R at the current column, clamped
+#pragma unroll
+    for (int i = 0; i < R + 2; ++i) {
+        int yy = y - 1 + i;
+        yy = yy < 0 ? 0 : (yy < h ? yy : h - 1);
+        yy = yy > y_end ? y_end : yy;   // rows no output needs may not be held (bands)
+        src[i] = in0 + ((u64)(yy - row0) * w * C + ch) * 2 * LIMBS * n + (u64)b * LIMBS * n + c;
+    }
+    u64* o = out0 + ((u64)(y - yout0) * w * C + ch) * 2 * (LIMBS - 1) * n + (u64)b * (LIMBS - 1) * n + c;
+    const u64 out_row = (u64)w * out_step;
+    u64 last[R][LIMBS], two[R][LIMBS];   // column sums: the last, and the last two
+    u64 raw[R + 2][LIMBS];               // the next column, loaded while the one before is worked on
+    auto load = [&] {
+#pragma unroll
+        for (int l = 0; l < LIMBS; ++l)
+#pragma unroll
+            for (int i = 0; i < R + 2; ++i) raw[i][l] = __ldg(src[i] + l * n);
+    };
+    auto advance = [&](int x) {          // raw = column x, or the last one again
+        if (x < w) {
+#pragma unroll
+            for (int i = 0; i < R + 2; ++i) src[i] += in_step;
+        }
+        load();
+    };
+    load();
+#pragma unroll
+    for (int r = 0; r < R; ++r)
 #pragma unroll
         for (int l = 0; l < LIMBS; ++l) {
-            ulonglong2 v0 = __ldg(r0 + off + l * half);
-            ulonglong2 v1 = __ldg(r1 + off + l * half);
-            ulonglong2 v2 = __ldg(r2 + off + l * half);
-            dst[l].x = v0.x + v1.x + v2.x;
-            dst[l].y = v0.y + v1.y + v2.y;
+            last[r][l] = raw[r][l] + raw[r + 1][l] + raw[r + 2][l];
+            two[r][l] = last[r][l] + last[r][l];   // x = -1 clamps to 0
         }
-    };
-    column(0, col[0]);  // x = -1 clamps to 0
-#pragma unroll
-    for (int l = 0; l < LIMBS; ++l) col[1][l] = col[0][l];
-    column(w > 1 ? 1 : 0, col[2]);
+    advance(1);
     for (int x = 0; x < w; ++x, o += out_step) {
-        mf_store<LIMBS>(a, col[0], col[1], col[2], o, half);
-        if (x + 1 < w) {
+        u64 sum[R][LIMBS];
 #pragma unroll
-            for (int l = 0; l < LIMBS; ++l) { col[0][l] = col[1][l]; col[1][l] = col[2][l]; }
-            column(x + 2 < w ? x + 2 : w - 1, col[2]);
-        }
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int l = 0; l < LIMBS; ++l) {
+                const u64 next = raw[r][l] + raw[r + 1][l] + raw[r + 2][l];
+                sum[r][l] = two[r][l] + next;
+                two[r][l] = last[r][l] + next;
+                last[r][l] = next;
+            }
+        if (x + 1 < w) advance(x + 2);
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            if (r == 0 || y + r < y_end) mf_store1<LIMBS>(a, sum[r], o + r * out_row, n);
     }
 }
 
@@ -378,7 +420,7 @@ __global__ void __launch_bounds__(256) k_meanfilter3_staged(const __grid_constan
     }
 }
 
-// Ragged batch, same items as k_meanfilter3_batch.
+// Ragged batch: segment s has h*chunks*2*c items, in the order of the single-image kernel.
 template <int LIMBS>
 __global__ void __launch_bounds__(512) k_meanfilter3_staged_batch(const __grid_constant__ OpsArgs a,
                                                                   const __grid_constant__ SegTable t)
@@ -403,47 +445,33 @@ __global__ void __launch_bounds__(512) k_meanfilter3_staged_batch(const __grid_c
     }
 }
 
-// One block per (row y, coefficient chunk, poly, channel); registers bounded so that three
-// blocks (up to three limbs) or two share an SM.
-template <int LIMBS>
-static constexpr int kMfMinBlocks = LIMBS <= 3 ? 3 : 2;
-
-template <int LIMBS>
-__global__ void __launch_bounds__(256, kMfMinBlocks<LIMBS>) k_meanfilter3(const __grid_constant__ OpsArgs a)
+// Ragged batch (a single image or a band of rows is a batch of one): segment s has
+// ceil(rows / R) * chunks * 2 * c items, row groups fastest, so that neighbouring blocks share their
+// halo rows in L2. Launched with at most 512 threads (the tunable shapes).
+template <int LIMBS, class Table>
+__global__ void __launch_bounds__(512) k_meanfilter3(const __grid_constant__ OpsArgs a, const __grid_constant__ Table t)
 {
-    const int chunks = ((1 << a.logn) / 2) / blockDim.x;
-    u64 bid = blockIdx.x;
-    const int y = a.y0 + (int)(bid % a.rows); bid /= a.rows;
-    const int chunk = (int)(bid % chunks); bid /= chunks;
-    const int b = (int)(bid % 2); bid /= 2;
-    meanfilter_row<LIMBS>(a, a.in0, a.out, a.h, a.w, a.c, y, chunk, b, (int)bid, a.row0, a.y0);
-}
-
-// Largest block of the batched mean-filter kernels for a limb count: the column sums of more
-// than three limbs need more than the 64 registers a thread gets at 1024 threads.
-template <int LIMBS>
-static constexpr int kMfMaxThreads = LIMBS <= 3 ? 1024 : 512;
-
-// Ragged batch: segment s has h*chunks*2*c items, in the order of the single-image kernel.
-// Launched with at most 512 threads (the tunable shapes).
-template <int LIMBS>
-__global__ void __launch_bounds__(kMfMaxThreads<LIMBS>) k_meanfilter3_batch(const __grid_constant__ OpsArgs a,
-                                                            const __grid_constant__ SegTable t)
-{
-    const int chunks = ((1 << a.logn) / 2) / blockDim.x;
+    constexpr int R = kMfRows<LIMBS>;
+    const int chunks = (1 << a.logn) / blockDim.x;
     const u64 total = t.start[t.n];
     for (u64 g = blockIdx.x; g < total; g += gridDim.x) {
         const int s = seg_of(t, g);
         u64 i = g - t.start[s];
         const int h = (int)t.h[s];
         const int rows = t.rows[s] ? (int)t.rows[s] : h;
-        const int y = (int)t.y0[s] + (int)(i % rows); i /= rows;
+        const int groups = (rows + R - 1) / R;
+        const int y0 = (int)t.y0[s], y = y0 + (int)(i % groups) * R; i /= groups;
         const int chunk = (int)(i % chunks); i /= chunks;
         const int b = (int)(i % 2); i /= 2;
-        meanfilter_row<LIMBS>(a, t.in0[s], t.out[s], h, (int)t.w[s], (int)t.c[s], y, chunk, b, (int)i, (int)t.row0[s],
-                              (int)t.y0[s]);
+        meanfilter_rows<LIMBS>(a, t.in0[s], t.out[s], h, (int)t.w[s], (int)t.c[s], y, y0 + rows, chunk, b, (int)i,
+                               (int)t.row0[s], y0);
     }
 }
+
+// Largest block of the fused kernel for a limb count: the column sums of more than three limbs need
+// more than the 64 registers a thread gets at 1024 threads.
+template <int LIMBS>
+static constexpr int kMfMaxThreads = LIMBS <= 3 ? 1024 : 512;
 
 // Fused radix encryption + 3x3 mean filter (Sec. 3.2, 3.3 and 4.4.1) for a ragged batch. Each
 // item is a strip of columns of one image for one polynomial, channel and 32 coefficient
@@ -975,6 +1003,13 @@ cudaError_t launch_rescale(const OpsArgs& a, cudaStream_t st)
     return cudaGetLastError();
 }
 
+static unsigned persistent_grid(u64 total, LaunchShape ls, int num_sms)
+{
+    // blocks_per_sm = 0: one block per work item (no grid-stride loop), capped at 2^31 - 1
+    const u64 cap = ls.blocks_per_sm > 0 ? (u64)num_sms * ls.blocks_per_sm : 0x7fffffffull;
+    return (unsigned)(total < cap ? total : cap);
+}
+
 // Launch of a staged mean-filter kernel: persistent grid of the blocks that fit on the GPU
 // (bounded by blocks_per_sm when it is set), dynamic shared memory for the two stages.
 template <typename K, typename... Args>
@@ -1002,14 +1037,47 @@ static int mf_staged_threads(int limbs, int threads)
     return threads;
 }
 
+template <class Table>
+static cudaError_t mf_launch(const OpsArgs& a, const Table& t, LaunchShape ls, int num_sms, cudaStream_t st)
+{
+    const unsigned g = persistent_grid(t.start[t.n], ls, num_sms);
+    if (g == 0) return cudaSuccess;
+    switch (a.limbs) {
+#define ICHEE_MF_CASE(LB) \
+    case LB: k_meanfilter3<LB, Table><<<g, ls.threads, 0, st>>>(a, t); break;
+        ICHEE_MF_CASE(2) ICHEE_MF_CASE(3) ICHEE_MF_CASE(4) ICHEE_MF_CASE(5) ICHEE_MF_CASE(6) ICHEE_MF_CASE(7) ICHEE_MF_CASE(8)
+#undef ICHEE_MF_CASE
+    default: return cudaErrorInvalidValue;
+    }
+    return cudaGetLastError();
+}
+
+static int mf_rows(int limbs)
+{
+    switch (limbs) {
+    case 2: return kMfRows<2>;
+    case 3: return kMfRows<3>;
+    case 4: return kMfRows<4>;
+    case 5: return kMfRows<5>;
+    case 6: return kMfRows<6>;
+    case 7: return kMfRows<7>;
+    default: return kMfRows<8>;
+    }
+}
+
+u64 mf_items(int logn, int limbs, int threads, bool staged, u32 rows, u32 c)
+{
+    if (staged) return (u64)rows * (((u64)1 << logn) / 2 / threads) * 2 * c;
+    const int r = mf_rows(limbs);
+    return ((u64)rows + r - 1) / r * (((u64)1 << logn) / threads) * 2 * c;
+}
+
 cudaError_t launch_meanfilter3(const OpsArgs& a, bool staged, int num_sms, cudaStream_t st)
 {
-    const int n = 1 << a.logn;
-    const int threads = 256;
-    const int chunks = (n / 2) / threads;
-    const u64 blocks = (u64)a.rows * chunks * 2 * a.c;
-    if (blocks == 0) return cudaSuccess;
+    const int threads = staged ? 256 : 128;   // 128: finer last waves on small images (256: 2 to 5 % slower there)
     if (staged) {
+        const u64 blocks = mf_items(a.logn, a.limbs, threads, true, (u32)a.rows, (u32)a.c);
+        if (blocks == 0) return cudaSuccess;
         switch (a.limbs) {
 #define ICHEE_MF_STAGED_CASE(LB) \
     case LB: return mf_staged_launch(k_meanfilter3_staged<LB>, LB, threads, blocks, 0, num_sms, st, a);
@@ -1019,28 +1087,19 @@ cudaError_t launch_meanfilter3(const OpsArgs& a, bool staged, int num_sms, cudaS
         default: return cudaErrorInvalidValue;
         }
     }
-    if (a.limbs >= 5) {
-        // five limbs and more through the batched kernel as a one-image batch (band included):
-        // it filters at 0.81 of copy bandwidth against 0.72 for the single-image kernel with the
-        // same launch shape, instruction count and traffic (fewer load stalls); at three limbs
-        // the single-image kernel is the faster one (0.75 against 0.70), at four they are level
-        SegTable t;
-        std::memset(&t, 0, sizeof(t));
-        t.n = 1;
-        t.start[0] = 0;
-        t.start[1] = blocks;
-        t.in0[0] = a.in0;
-        t.out[0] = a.out;
-        t.h[0] = (uint32_t)a.h;
-        t.w[0] = (uint32_t)a.w;
-        t.c[0] = (uint32_t)a.c;
-        t.y0[0] = (uint32_t)a.y0;
-        t.rows[0] = (uint32_t)a.rows;
-        t.row0[0] = (uint32_t)a.row0;
-        return launch_meanfilter3_batch(a, t, LaunchShape{threads, 0}, false, num_sms, st);
-    }
-    ICHEE_LIMB_SWITCH(k_meanfilter3, (unsigned)blocks, threads, a)
-    return cudaGetLastError();
+    OneSeg t;   // the image, or its band, as a batch of one
+    std::memset(&t, 0, sizeof(t));
+    t.n = 1;
+    t.start[1] = mf_items(a.logn, a.limbs, threads, false, (u32)a.rows, (u32)a.c);
+    t.in0[0] = a.in0;
+    t.out[0] = a.out;
+    t.h[0] = (uint32_t)a.h;
+    t.w[0] = (uint32_t)a.w;
+    t.c[0] = (uint32_t)a.c;
+    t.y0[0] = (uint32_t)a.y0;
+    t.rows[0] = (uint32_t)a.rows;
+    t.row0[0] = (uint32_t)a.row0;
+    return mf_launch(a, t, LaunchShape{threads, 0}, num_sms, st);
 }
 
 cudaError_t launch_blend(const OpsArgs& a, cudaStream_t st)
@@ -1057,13 +1116,6 @@ cudaError_t launch_blend(const OpsArgs& a, cudaStream_t st)
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
-}
-
-static unsigned persistent_grid(u64 total, LaunchShape ls, int num_sms)
-{
-    // blocks_per_sm = 0: one block per work item (no grid-stride loop), capped at 2^31 - 1
-    const u64 cap = ls.blocks_per_sm > 0 ? (u64)num_sms * ls.blocks_per_sm : 0x7fffffffull;
-    return (unsigned)(total < cap ? total : cap);
 }
 
 cudaError_t launch_meanfilter3_batch(const OpsArgs& a, const SegTable& t, LaunchShape ls, bool staged, int num_sms,
@@ -1085,9 +1137,7 @@ cudaError_t launch_meanfilter3_batch(const OpsArgs& a, const SegTable& t, Launch
         default: return cudaErrorInvalidValue;
         }
     }
-    const unsigned g = persistent_grid(total, ls, num_sms);
-    ICHEE_LIMB_SWITCH_T(k_meanfilter3_batch, g, ls.threads, a, t)
-    return cudaGetLastError();
+    return mf_launch(a, t, ls, num_sms, st);
 }
 
 // Threads per block of the fused kernel for a launch shape: 32 x columns per strip (at least 4

@@ -74,8 +74,10 @@ cudaError_t launch_decrypt(const DecArgs& a, int threads, cudaStream_t st);
 cudaError_t launch_meanfilter3_batch(const OpsArgs& a, const SegTable& t, LaunchShape ls, bool staged, int num_sms,
                                      cudaStream_t st);
 // Threads per block the batched mean filter runs with for a requested count (the staged form
-// halves it while its stages would not fit); items are counted with it.
+// halves it while its stages would not fit), and the items of an image (or of a band of rows) with
+// that many threads.
 int mf_batch_threads(int limbs, int threads, bool staged);
+u64 mf_items(int logn, int limbs, int threads, bool staged, u32 rows, u32 c);
 cudaError_t launch_blend_batch(const OpsArgs& a, const SegTable& t, LaunchShape ls, int num_sms, cudaStream_t st);
 cudaError_t launch_ptadd_batch(const OpsArgs& a, const SegTable& t, LaunchShape ls, int num_sms, cudaStream_t st);
 cudaError_t launch_decrypt_batch(const DecArgs& a, const SegTable& t, LaunchShape ls, int num_sms, cudaStream_t st);
