@@ -18,8 +18,9 @@ struct EncShape {
     static constexpr int T = N / E;
     static constexpr int NP = LOGN <= 13 ? 2 : 1;
     static constexpr int KEEP = 2;   // v^ modulo two primes at a time
+    static constexpr int BUFS = LOGN <= 13 ? 2 : 1;   // exchange buffers, used in turn (two do not fit at 2^14)
     static constexpr int BLOCKS = 1024 / T;
-    static constexpr size_t CDT_AT = (size_t)N * (4 * NP + 4 * KEEP + 2);
+    static constexpr size_t CDT_AT = (size_t)N * (4 * NP * BUFS + 4 * KEEP + 2);
     static constexpr size_t SMEM = CDT_AT + 32 * sizeof(u64);
     static_assert(SMEM <= 227 * 1024 && BLOCKS * (SMEM + 1024) <= 228 * 1024, "shared memory of an SM");
 };
@@ -366,8 +367,8 @@ __device__ __forceinline__ void encrypt_ct(const EncArgs& a, int p, u64 seed, u6
 {
     using S = EncShape<LOGN>;
     constexpr int N = 1 << LOGN, E = S::E, T = S::T, NP = S::NP, LAST = NttShape<LOGN, E>::LAST;
-    u32* ex = reinterpret_cast<u32*>(smem);                       // exchange buffer, N words of 4 NP bytes
-    u32* vh = ex + NP * N;                                        // v^ modulo S::KEEP primes, thread-major
+    u32* ex = reinterpret_cast<u32*>(smem);                       // exchange buffers, N words of 4 NP bytes
+    u32* vh = ex + S::BUFS * NP * N;                                        // v^ modulo S::KEEP primes, thread-major
     uint16_t* smp = reinterpret_cast<uint16_t*>(vh + S::KEEP * N);
     const u64* tcdt = reinterpret_cast<const u64*>(reinterpret_cast<unsigned char*>(smem) + S::CDT_AT);
     const int tid = threadIdx.x;
@@ -392,19 +393,26 @@ __device__ __forceinline__ void encrypt_ct(const EncArgs& a, int p, u64 seed, u6
 
     const int x0 = elem_index<LOGN, 0, E>(tid, 0);       // first-pass layout: x0 + elem_offset(e)
     const int xl = elem_index<LOGN, LAST, E>(tid, 0);    // last-pass layout
+    // Up to N = 2^13 the transforms alternate two exchange buffers and need no barrier between them: a
+    // transform's exchanges make every warp wait, through the groups that trade data, for all others,
+    // so a buffer's earlier loads are over when it is written again (checked for every ring in the
+    // host-compiled test of the groups). One buffer and a block barrier before each transform: 2.3 %
+    // slower.
     // First the third prime, for the limbs that need it: its digits wait in the output's own words
     // (each thread's coefficients of the ciphertext, which it overwrites with the residues below),
     // so that at most two primes' digits are in registers. Then the first two primes of every limb.
+    int turn = 0;
 #pragma unroll 1
     for (int phase = a.aux.n == 3 ? 0 : 1; phase < 2; ++phase) {
         const int i0 = phase == 0 ? 2 : 0, i1 = phase == 0 ? 3 : 2;
 #pragma unroll 1
         for (int i = i0; i < i1; ++i) {
-            __syncthreads();   // the exchange buffer's last readers are done
+            __syncthreads();   // samples drawn; the exchange buffer's last readers are done
             u32 r[1][E];
 #pragma unroll
             for (int e = 0; e < E; ++e) r[0][e] = (u32)((int)(smp[x0 + elem_offset<LOGN, 0, E>(e)] & 3u) - 1);
-            ntt32_fwd<LOGN, 1, E, true>(ex, r, tid, a.aux.tw[i], a.aux.p[i]);
+            ntt32_fwd<LOGN, 1, E, true>(ex + (S::BUFS == 2 ? turn * NP * N : 0), r, tid, a.aux.tw[i], a.aux.p[i]);
+            turn ^= 1;
 #pragma unroll
             for (int e = 0; e < E; ++e) vh[(i - i0) * N + e * T + tid] = r[0][e];
         }
@@ -435,8 +443,9 @@ __device__ __forceinline__ void encrypt_ct(const EncArgs& a, int p, u64 seed, u6
                             y[0][e] = mont32(v, __ldg(pk + o), pi, pinv);
                         }
                     }
-                    __syncthreads();
-                    ntt32_inv<LOGN, NP, E>(ex, y, tid, a.aux.itw[i], pi);
+                    if (S::BUFS == 1) __syncthreads();
+                    ntt32_inv<LOGN, NP, E>(ex + (S::BUFS == 2 ? turn * NP * N : 0), y, tid, a.aux.itw[i], pi);
+                    turn ^= 1;
                 }
                 u64* dst = ct + ((u64)pb * L + l) * N + x0;
                 if (phase == 0) {

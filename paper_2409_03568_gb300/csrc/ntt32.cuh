@@ -149,7 +149,7 @@ __device__ __forceinline__ void fwd32_rest(u32* sm, u32 (&r)[NP][E], int tid, co
     constexpr int LE = Radix<E>::LE;
     if constexpr (S0 <= NttShape<LOGN, E>::LAST) {
         store_sm32<LOGN, S0 - LE, NP, E>(sm, r, tid);
-        exchange_barrier<exchange_in_warp(LOGN, S0 - LE, S0, E)>();
+        exchange_barrier<LOGN, S0, E>();
         load_sm32<LOGN, S0, NP, E>(sm, r, tid);
         fwd32_regs<LOGN, S0, NP, E, B, false>(r, tid, tw, p);
         fwd32_rest<LOGN, S0 + LE, NP, E, fwd32_bound(B, Pass<LOGN, S0, E>::S)>(sm, r, tid, tw, p);
@@ -240,7 +240,7 @@ __device__ __forceinline__ void inv32_rest(u32* sm, u32 (&r)[NP][E], int tid, co
     inv32_regs<LOGN, S0, NP, E, B>(r, tid, itw, p);
     if constexpr (S0 > 0) {
         store_sm32<LOGN, S0, NP, E>(sm, r, tid);
-        exchange_barrier<exchange_in_warp(LOGN, S0, S0 - LE, E)>();
+        exchange_barrier<LOGN, S0, E>();
         load_sm32<LOGN, S0 - LE, NP, E>(sm, r, tid);
         inv32_rest<LOGN, S0 - LE, NP, E, inv32_bound(B, Pass<LOGN, S0, E>::S)>(sm, r, tid, itw, p);
     }
