@@ -738,6 +738,82 @@ __global__ void __launch_bounds__(256, LIMBS <= 5 ? 3 : 2) k_blend_wide(const __
     blend_rows<LIMBS>(a);
 }
 
+// A one-channel pattern under an image of C > 1 channels: a thread takes one coefficient of a pixel
+// for all its channels, so the pattern's residues are loaded, and their products made, once instead
+// of per channel; the next channel's residues are loaded before the current channel's products.
+// Work unit: (pixel, polynomial, share of the coefficients). From four limbs up: 97x61x3 at N = 2^13
+// 3.46 -> 3.20 ms (6.05 TB/s, pattern counted once), 48x48x3 at N = 2^14 and five limbs 3.35 -> 3.07
+// ms; with three limbs k_blend's 16-byte loads are the faster form (2.44 against 2.53 ms).
+template <int LIMBS>
+__global__ void __launch_bounds__(256, LIMBS <= 5 ? 4 : 2) k_blend_shared(const __grid_constant__ OpsArgs a, int splits)
+{
+    constexpr int t = LIMBS - 1;
+    const int n = 1 << a.logn, span = n / splits;
+    const u64 qt = a.q[t];
+    const u64 units = a.n_ct / a.c * 2 * splits;
+    const u64 in_ch = (u64)2 * LIMBS * n, out_ch = (u64)2 * (LIMBS - 1) * n;   // to the next channel
+    for (u64 u = blockIdx.x; u < units; u += gridDim.x) {
+        const u64 px = u / (2 * splits);
+        const int b = (int)(u / splits) & 1;
+        const u64 from = (u64)(u % splits) * span;
+        for (int c = threadIdx.x; c < span; c += blockDim.x) {
+            const u64* ci = a.in0 + px * a.c * in_ch + (u64)b * LIMBS * n + from + c;
+            const u64* cw = a.in1 + px * in_ch + (u64)b * LIMBS * n + from + c;
+            u64* co = a.out + px * a.c * out_ch + (u64)b * (LIMBS - 1) * n + from + c;
+            u64 x[LIMBS], w[LIMBS];
+#pragma unroll
+            for (int l = 0; l < LIMBS; ++l) w[l] = __ldcs(cw + l * n);
+#pragma unroll
+            for (int l = 0; l < LIMBS; ++l) x[l] = __ldcs(ci + l * n);
+            // the pattern's share of every channel (as in blend_pair)
+            const u64 wt = w[t];
+            u64 hw = 0, rw;
+            if (a.k01_same) {
+                hw = mulhi(wt, a.k1p[t]);
+                rw = wt * a.k1[t] - hw * qt;
+            } else {
+                rw = shoup(wt, a.k1[t], a.k1p[t], qt);
+            }
+#pragma unroll
+            for (int j = 0; j < t; ++j)
+                w[j] = shoup_lazy(a.k01_same ? w[j] + a.mq[j] - wt : w[j], a.k1r[j], a.k1rp[j], a.q[j]);
+            for (int ch = 0; ch < a.c; ++ch, co += out_ch) {
+                u64 next[LIMBS];
+                if (ch + 1 < a.c) {
+                    ci += in_ch;
+#pragma unroll
+                    for (int l = 0; l < LIMBS; ++l) next[l] = __ldcs(ci + l * n);
+                }
+                const u64 xt = x[t];
+                if (a.k01_same) {
+                    const u64 hx = mulhi(xt, a.k0p[t]);
+                    u64 r = (xt * a.k0[t] - hx * qt) + rw;   // in [0, 4 q_t)
+                    u64 q = hx + hw;
+                    if (r >= 2 * qt) { r -= 2 * qt; q += 2; }
+                    if (r >= qt) { r -= qt; q += 1; }
+                    q += r > a.half_qt ? 1 : 0;
+#pragma unroll
+                    for (int j = 0; j < t; ++j) {
+                        const u64 qj = a.q[j];
+                        u64 v = shoup_lazy(x[j] + a.mq[j] - xt, a.k0r[j], a.k0rp[j], qj) + w[j] + csub_s(q, qj);
+                        v = csub_s(csub_s(v, 4 * qj), 2 * qj);   // from [0, 5 q_j)
+                        __stcs(co + j * n, csub_s(v, qj));
+                    }
+                } else {
+                    const u64 tt = add_mod(shoup(xt, a.k0[t], a.k0p[t], qt), rw, qt);
+#pragma unroll
+                    for (int j = 0; j < t; ++j) {
+                        const u64 v = csub_s(shoup_lazy(x[j], a.k0r[j], a.k0rp[j], a.q[j]) + w[j], 2 * a.q[j]);
+                        __stcs(co + j * n, rescale_fold(v, tt, j, a));
+                    }
+                }
+#pragma unroll
+                for (int l = 0; l < LIMBS; ++l) x[l] = next[l];
+            }
+        }
+    }
+}
+
 // Ragged batch: one block of kBlendBatchThreads per ciphertext; W of segment s has c1[s]
 // channels. Compiled for three blocks per SM up to five limbs, as the single-image kernel.
 constexpr int kBlendBatchThreads = 256;
@@ -1104,6 +1180,22 @@ cudaError_t launch_meanfilter3(const OpsArgs& a, bool staged, int num_sms, cudaS
 
 cudaError_t launch_blend(const OpsArgs& a, cudaStream_t st)
 {
+    if (a.limbs >= 4 && a.c_w == 1 && a.c > 1) {   // both forms measured at k_blend_shared
+        // coefficients shared out until the grid has a few blocks per SM
+        const u64 px2 = a.n_ct / a.c * 2;
+        int splits = 1;
+        while (px2 * splits < 152 * 16 && ((1 << a.logn) / splits) > 256) splits *= 2;
+        const u64 units = px2 * splits;
+        const unsigned g = (unsigned)(units < (1u << 30) ? units : (1u << 30));
+        switch (a.limbs) {
+#define ICHEE_BLEND_CASE(LB) \
+    case LB: k_blend_shared<LB><<<g, 256, 0, st>>>(a, splits); break;
+            ICHEE_BLEND_CASE(4) ICHEE_BLEND_CASE(5) ICHEE_BLEND_CASE(6) ICHEE_BLEND_CASE(7) ICHEE_BLEND_CASE(8)
+#undef ICHEE_BLEND_CASE
+        default: return cudaErrorInvalidValue;
+        }
+        return cudaGetLastError();
+    }
     const unsigned g = grid_for(2 * a.n_ct, 1);   // rows (ciphertext, polynomial)
     switch (a.limbs) {
     case 2: k_blend<2><<<g, 256, 0, st>>>(a); break;
