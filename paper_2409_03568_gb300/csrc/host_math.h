@@ -22,7 +22,22 @@ inline u64 powm(u64 base, u64 exp, u64 m)
     return acc;
 }
 
-inline u64 invm(u64 a, u64 p) { return powm(a, p - 2, p); }  // p prime
+// a^{-1} mod p for a prime to p < 2^62 (extended Euclid: some 35 divisions; operations take several
+// inverses per call, and a power by square and multiply took ten times as long).
+inline u64 invm(u64 a, u64 p)
+{
+    u64 r0 = p, r1 = a % p;
+    int64_t t0 = 0, t1 = 1;
+    while (r1 != 0) {
+        const u64 quo = r0 / r1, r2 = r0 - quo * r1;
+        const int64_t t2 = t0 - (int64_t)quo * t1;
+        r0 = r1;
+        r1 = r2;
+        t0 = t1;
+        t1 = t2;
+    }
+    return t0 < 0 ? (u64)(t0 + (int64_t)p) : (u64)t0;
+}
 
 // Strong-probable-prime test to the first twelve prime bases (exact below 2^64).
 inline bool is_prime64(u64 n)

@@ -214,33 +214,9 @@ extern "C" ichee_status ichee_ctx_create(const ichee_params* p, int device, iche
         c->rns.tab[m].tw = reinterpret_cast<const ulonglong2*>(base);
         c->rns.tab[m].itw = reinterpret_cast<const ulonglong2*>(base + 2 * (size_t)c->n);
         ninv[m] = hm::invm((u64)c->n % qm, qm);
-        if (sqdiff_split(c->logn)) {   // twiddles of the two half transforms after the first stage
-            const size_t nh = (size_t)c->n / 2;
-            if (!c->d_half_tw && cudaMalloc(&c->d_half_tw, (size_t)c->nmod * 4 * nh * 8) != cudaSuccess)
-                return cleanup(fail(ICHEE_ENOMEM, "half tables"));
-            std::vector<u64> half(4 * nh, 0);
-            for (int h = 0; h < 2; ++h)
-                for (size_t k = 1; k < nh; ++k) {
-                    size_t s2 = 1;
-                    while (s2 * 2 <= k) s2 *= 2;
-                    const size_t src = (2 + h) * s2 + (k - s2);
-                    half[((size_t)h * nh + k) * 2] = t[src];
-                    half[((size_t)h * nh + k) * 2 + 1] = t[(size_t)c->n + src];
-                }
-            u64* hb = c->d_half_tw + (size_t)m * 4 * nh;
-            if (cudaMemcpy(hb, half.data(), half.size() * 8, cudaMemcpyHostToDevice) != cudaSuccess)
-                return cleanup(fail(ICHEE_ECUDA, "upload half tables"));
-            for (int h = 0; h < 2; ++h) {
-                c->half_tab[h][m].tw = reinterpret_cast<const ulonglong2*>(hb + (size_t)h * 2 * nh);
-                c->half_tab[h][m].itw = nullptr;
-            }
-        }
     }
-    if (cudaMalloc(&c->d_ninv, 16 * (size_t)c->nmod) != cudaSuccess) return cleanup(fail(ICHEE_ENOMEM, "ninv"));
-    for (int m = 0; m < c->nmod; ++m)   // N^{-1} 2^64: undoes a Montgomery product's 2^{-64} as well
-        ninv.push_back(hm::mulm(ninv[m], (u64)(((hm::u128)1 << 64) % c->q[m]), c->q[m]));
-    cudaMemcpy(c->d_ninv, ninv.data(), 16 * (size_t)c->nmod, cudaMemcpyHostToDevice);
-    c->d_ninv_r = c->d_ninv + c->nmod;
+    if (cudaMalloc(&c->d_ninv, 8 * (size_t)c->nmod) != cudaSuccess) return cleanup(fail(ICHEE_ENOMEM, "ninv"));
+    cudaMemcpy(c->d_ninv, ninv.data(), 8 * (size_t)c->nmod, cudaMemcpyHostToDevice);
 
     // Delta * p mod q_l for p = 0..255
     std::vector<u64> dm((size_t)c->L * 256);
@@ -292,7 +268,7 @@ extern "C" void ichee_ctx_destroy(ichee_ctx* c)
     if (!c) return;
     cudaSetDevice(c->device);
     cudaDeviceSynchronize();
-    void* ptrs[] = {c->d_tables, c->d_half_tw, c->d_dm, c->d_ninv, c->d_s, c->d_srev, c->d_pk, c->d_aux_tables, c->d_pk_aux,
+    void* ptrs[] = {c->d_tables, c->d_dm, c->d_ninv, c->d_s, c->d_srev, c->d_pk, c->d_aux_tables, c->d_pk_aux,
                     c->d_evk, c->d_evk_hat, c->d_evk_hat_p, c->d_status};
     for (void* p : ptrs)
         if (p) cudaFree(p);
@@ -1272,7 +1248,7 @@ static int sqdiff_blocks(const ichee_ctx* c, int limbs, u64 n_ct)
 static size_t sqdiff_slice_words(const ichee_ctx* c) { return (size_t)(sqdiff_split(c->logn) ? 2 : 4) * c->n; }
 
 // Words of the relinearisation working set: the tensor [3][limbs][N], the key-switching digits,
-// the accumulators over Q*P and the relinearised pair.
+// the accumulators over Q*P and t2 in the coefficient domain (in the room of a ciphertext).
 static size_t relin_words(const ichee_ctx* c, int limbs)
 {
     const size_t n = (size_t)c->n;
@@ -1296,60 +1272,60 @@ static ichee_status sqdiff_partial_sum(ichee_ctx* c, const uint64_t* d_a, const 
     sa.b = d_b;
     sa.partial = partial;
     sa.n_blocks = n_blocks;
-    for (int h = 0; h < 2; ++h)
-        for (int l = 0; l < limbs; ++l) sa.htab[h][l] = c->half_tab[h][l];
     CK(launch_sqdiff_accumulate(sa, st));
     CK(launch_sqdiff_reduce(sa.rns, limbs, partial, n_blocks, tensor, add, st));
     return ICHEE_OK;
 }
 
-// tensor (reduced residues, NTT domain, overwritten) -> INTT -> relinearise -> rescale into
+// Keys and constants of relinearisation and rescale at a level (everything but inputs and outputs).
+static SqImgArgs relin_args(const ichee_ctx* c, int limbs)
+{
+    const int t = limbs - 1;
+    SqImgArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.rns = c->rns;
+    a.L = c->L;
+    a.limbs = limbs;
+    a.evk_hat = c->d_evk_hat;
+    a.evk_hat_p = c->d_evk_hat_p;
+    const u64 qt = c->q[t];
+    a.half_qt = (qt - 1) / 2;
+    for (int j = 0; j < limbs; ++j) {
+        const u64 qj = c->q[j];
+        const u64 r64 = (u64)(((hm::u128)1 << 64) % qj);   // undoes the tensor's Montgomery 2^{-64}
+        a.ninv[j] = hm::mulm(hm::invm((u64)c->n % qj, qj), r64, qj);
+        a.ninv_p[j] = hm::shoup_of(a.ninv[j], qj);
+        a.pn[j] = hm::mulm(c->P % qj, a.ninv[j], qj);
+        a.pn_p[j] = hm::shoup_of(a.pn[j], qj);
+        a.r64[j] = r64;
+        a.r64_p[j] = hm::shoup_of(r64, qj);
+        a.p_inv[j] = hm::invm(c->P % qj, qj);
+        a.p_inv_p[j] = hm::shoup_of(a.p_inv[j], qj);
+        const u64 r = c->P % qj;
+        a.neg_p_mod[j] = r == 0 ? 0 : qj - r;
+        if (j < t) {
+            a.qt_inv[j] = hm::invm(qt % qj, qj);
+            a.qt_inv_p[j] = hm::shoup_of(a.qt_inv[j], qj);
+        }
+    }
+    return a;
+}
+
+// tensor (reduced residues, NTT domain) -> relinearise -> rescale into
 // d_out (one ciphertext at level - 1). work: relin_words - 3 limbs N words after the tensor.
 static ichee_status sqdiff_relin_rescale(ichee_ctx* c, u64* tensor, const ichee_ctimg_meta* ma, u64* work,
                                          uint64_t* d_out, ichee_ctimg_meta* mout, cudaStream_t st)
 {
     const int limbs = (int)ma->level + 1;
     const size_t n = (size_t)c->n;
-    const int L = c->L;
     u64* digits = work;
     u64* acc = digits + (size_t)limbs * (limbs + 1) * n;
-    u64* rel = acc + (size_t)2 * (limbs + 1) * n;
-    int id[kMaxModuli];
-    for (int m = 0; m < kMaxModuli; ++m) id[m] = m;
-    CK(launch_ntt_inv(c->rns, batch(tensor, 3 * limbs, limbs, id), st));
-    CK(launch_scale_const(c->rns, batch(tensor, 3 * limbs, limbs, id), c->d_ninv_r, st));
-
-    RelinArgs ra;
-    std::memset(&ra, 0, sizeof(ra));
-    ra.rns = c->rns;
-    ra.L = L;
-    ra.limbs = limbs;
-    ra.evk_hat = c->d_evk_hat;
-    ra.evk_hat_p = c->d_evk_hat_p;
-    for (int m = 0; m < c->nmod; ++m) ra.mu[m] = c->rns.mu[m];
-    for (int j = 0; j < limbs; ++j) {
-        ra.p_inv[j] = hm::invm(c->P % c->q[j], c->q[j]);
-        ra.p_inv_p[j] = hm::shoup_of(ra.p_inv[j], c->q[j]);
-        const u64 r = c->P % c->q[j];
-        ra.neg_p_mod[j] = r == 0 ? 0 : c->q[j] - r;
-    }
-    int midx[kMaxModuli];
-    for (int m = 0; m < limbs; ++m) midx[m] = m;
-    midx[limbs] = L;
-    CK(launch_relin_digits(ra, tensor + (size_t)2 * limbs * n, digits, st));
-    CK(launch_ntt_fwd(c->rns, batch(digits, limbs * (limbs + 1), limbs + 1, midx), st));
-    CK(launch_relin_mac(ra, digits, acc, st));
-    CK(launch_ntt_inv(c->rns, batch(acc, 2 * (limbs + 1), limbs + 1, midx), st));
-    CK(launch_relin_moddown(ra, tensor, acc, rel, st));
-
-    ichee_ctimg_meta one = *ma;
-    one.h = one.w = one.c = 1;
-    OpsArgs a = ops_base(c, &one);
-    a.in0 = rel;
+    u64* t2 = acc + (size_t)2 * (limbs + 1) * n;
+    SqImgArgs a = relin_args(c, limbs);
     a.out = d_out;
-    set_rescale(c, a);
-    CK(launch_rescale(a, st));
-    *mout = one;
+    CK(launch_relin_rescale(a, tensor, t2, digits, acc, st));
+    *mout = *ma;
+    mout->h = mout->w = mout->c = 1;
     mout->level = ma->level - 1;
     mout->scale = ma->scale * ma->scale / (double)c->q[ma->level];
     return ICHEE_OK;
@@ -1457,46 +1433,19 @@ static ichee_status op_sqdiff_image(ichee_ctx* c, const uint64_t* d_a, const ich
     if (!c->have_evk) return fail(ICHEE_EUNSUPPORTED, "squared difference needs the evaluation key (ICHEE_WITH_EVK)");
     if (ma->level == 0) return fail(ICHEE_ELEVEL, "squared difference needs a limb to drop");
     const int limbs = (int)ma->level + 1;
-    const int t = limbs - 1;
     const u64 n_ct = (u64)ma->h * ma->w * ma->c;
     const int grid = sqdiff_image_grid(c->logn, n_ct, c->num_sms);
     CK(c->scratch.ensure((size_t)grid * sqdiff_image_scratch_words(c->logn, limbs) * 8, c->user_alloc, c->user_free, c->user_alloc_ctx, st));
-    SqImgArgs a;
-    std::memset(&a, 0, sizeof(a));
-    a.rns = c->rns;
-    a.L = c->L;
-    a.limbs = limbs;
+    SqImgArgs a = relin_args(c, limbs);
     a.n_ct = n_ct;
     a.a = d_a;
     a.b = d_b;
     a.out = d_out;
     a.scratch = (u64*)c->scratch.p;
-    a.evk_hat = c->d_evk_hat;
-    a.evk_hat_p = c->d_evk_hat_p;
-    const u64 qt = c->q[t];
-    a.half_qt = (qt - 1) / 2;
-    for (int j = 0; j < limbs; ++j) {
-        const u64 qj = c->q[j];
-        const u64 r64 = (u64)(((hm::u128)1 << 64) % qj);   // undoes the tensor's Montgomery 2^{-64}
-        a.ninv[j] = hm::mulm(hm::invm((u64)c->n % qj, qj), r64, qj);
-        a.ninv_p[j] = hm::shoup_of(a.ninv[j], qj);
-        a.pn[j] = hm::mulm(c->P % qj, a.ninv[j], qj);
-        a.pn_p[j] = hm::shoup_of(a.pn[j], qj);
-        a.r64[j] = r64;
-        a.r64_p[j] = hm::shoup_of(r64, qj);
-        a.p_inv[j] = hm::invm(c->P % qj, qj);
-        a.p_inv_p[j] = hm::shoup_of(a.p_inv[j], qj);
-        const u64 r = c->P % qj;
-        a.neg_p_mod[j] = r == 0 ? 0 : qj - r;
-        if (j < t) {
-            a.qt_inv[j] = hm::invm(qt % qj, qj);
-            a.qt_inv_p[j] = hm::shoup_of(a.qt_inv[j], qj);
-        }
-    }
     CK(launch_sqdiff_image(a, grid, st));
     *mout = *ma;
     mout->level = ma->level - 1;
-    mout->scale = ma->scale * ma->scale / (double)qt;
+    mout->scale = ma->scale * ma->scale / (double)c->q[ma->level];
     return ICHEE_OK;
 }
 

@@ -110,9 +110,8 @@ __global__ void __launch_bounds__(NttShape<LOGN, E>::T, sqdiff_blocks_per_sm(LOG
 // takes limb j % limbs and half h = (j / limbs) % 2: it loads both halves of d = a - b, applies
 // the first-stage butterfly for its half only (the product W d_hi is made by both halves'
 // blocks: 1/14 more products), and runs the other 13 stages with the 2^13-point code -- 8
-// residues per thread, 1024 threads, no spills -- and the half's twiddles:
-// tw_h[2^s + g] = tw[(2 + h) 2^s + g]. Its tensor terms go to a [4][N/2] slice. The two
-// blocks of a half pair read the same ciphertexts at about the same time (one HBM read, one
+// residues per thread, 1024 threads, no spills -- from root 2 + h of the table. Its tensor terms go to
+// a [4][N/2] slice. The two blocks of a half pair read the same ciphertexts at about the same time (one HBM read, one
 // L2 hit).
 template <int CAP>
 __device__ __forceinline__ void sqdiff_accumulate_split(const SqDiffArgs& a, u64* buf)
@@ -130,7 +129,7 @@ __device__ __forceinline__ void sqdiff_accumulate_split(const SqDiffArgs& a, u64
     u64* acc = a.partial + (size_t)blockIdx.x * 4 * NH;
     const u64 q = a.rns.q[l];
     const u64 qinv = a.rns.qinv[l];
-    const ModTables t = a.htab[h][l];
+    const ModTables t = a.rns.tab[l];   // the halves' roots are 2 and 3
     const ulonglong2 w1 = a.rns.tab[l].tw[1];   // the first stage's twiddle and its companion
 #pragma unroll
     for (int e = 0; e < E; e += 2) {
@@ -157,7 +156,7 @@ __device__ __forceinline__ void sqdiff_accumulate_split(const SqDiffArgs& a, u64
             }
             if (pb == 0) __syncthreads();   // d0 in its parking buffer, d1 in the other (as above)
             u64* dst = pb == 0 ? d0buf : buf;
-            ntt_fwd_regs<LOGH, false, E, CAP, IN>(dst, r, tid, t, q);
+            ntt_fwd_regs<LOGH, false, E, CAP, IN>(dst, r, tid, t, q, 2 + h);
             const int sb = slot_base<LOGH, LAST, E>(tid);
 #pragma unroll
             for (int e = 0; e < E; ++e)
@@ -224,8 +223,16 @@ __global__ void k_sqdiff_reduce(RnsArgs rns, int limbs, const u64* partial, int 
     for (int x = blockIdx.x * blockDim.x + threadIdx.x; x < n; x += gridDim.x * blockDim.x) {
         u64 s = 0;
         const int h = split ? x / row : 0, xx = split ? x % row : x;
-        for (int j = l + h * limbs; j < n_blocks; j += step)   // slices in [0, 2q), the sum too
-            s = csub_s(s + partial[((size_t)j * 4 + p) * row + xx], 2 * q);
+        for (int j = l + h * limbs; j < n_blocks; j += 8 * step) {   // slices in [0, 2q), the sum too
+            u64 v[8];   // eight loads in flight
+#pragma unroll
+            for (int u = 0; u < 8; ++u) {
+                const int ju = j + u * step;
+                v[u] = ju < n_blocks ? partial[((size_t)ju * 4 + p) * row + xx] : 0;
+            }
+#pragma unroll
+            for (int u = 0; u < 8; ++u) s = csub_s(s + v[u], 2 * q);
+        }
         s = csub_s(s, q);
         if (p == 1) s = add_mod(s, s, q);                      // 2 d0 d1
         if (add) s = add_mod(s, reduce64(tensor[(size_t)pl * n + x], q, rns.mu[l]), q);
@@ -547,89 +554,188 @@ cudaError_t launch_sqdiff_image(const SqImgArgs& a, int grid, cudaStream_t st)
 }
 
 // ---------------------------------------------------------------------------------------
-// Relinearisation by hybrid key switching with one special prime P, one digit per ciphertext
-// prime, mod-down with centered rounding.
+// Relinearisation and rescale of one degree-2 ciphertext in the transform domain (matching's sum):
+// hybrid key switching with one special prime P, one digit per ciphertext prime, mod-down and
+// rescale with centered rounding, as the per-pixel kernel does them (t0^ and t1^ stay in the
+// transform domain, times P; digit j needs no transform into its own modulus). One ciphertext has
+// few transforms, so each is split over R = 2^LS blocks (R = 8; 4 at N = 2^10) -- the stages that
+// couple the parts run in the elementwise kernels before and after -- and lifts, key products,
+// mod-down and rescale ride along. Five short launches after the sum instead of eight with whole
+// transforms in one block each: 43 instead of 67 us of kernels at N = 2^13 and three limbs, 52 instead
+// of 119 at N = 2^14 and five; matching of one pair 116 -> 75 and 171 -> 89 us.
 // ---------------------------------------------------------------------------------------
+template <int LOGN>
+static constexpr int kRelinLs = LOGN == 10 ? 2 : 3;
 
-__global__ void k_relin_digits(const __grid_constant__ RelinArgs a, const u64* d2, u64* digits)
+// t2: the parts of INTT(t2^ N^{-1} 2^64) of every limb, below 4q. Block (limb, part).
+template <int LOGN>
+__global__ void __launch_bounds__((1 << (LOGN - kRelinLs<LOGN>)) / 8) k_relin_t2(const __grid_constant__ SqImgArgs a,
+                                                                               const u64* t2_hat, u64* t2)
 {
-    const int n = 1 << a.rns.logn;
+    constexpr int LS = kRelinLs<LOGN>, LOGM = LOGN - LS, E = 8, LAST = NttShape<LOGM, E>::LAST;
+    extern __shared__ u64 sm[];
+    const int tid = threadIdx.x, l = blockIdx.x >> LS, h = blockIdx.x & ((1 << LS) - 1);
+    const u64 q = a.rns.q[l];
+    const size_t at = ((size_t)l << LOGN) + ((size_t)h << LOGM);
+    u64 r[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+        r[e] = shoup3(t2_hat[at + elem_index<LOGM, LAST, E>(tid, e)], a.ninv[l], a.ninv_p[l], q);
+    ntt_inv_regs<LOGM, false, E, 8>(sm, r, tid, a.rns.tab[l], q, (1 << LS) + h);
+#pragma unroll
+    for (int e = 0; e < E; ++e) t2[at + elem_index<LOGM, 0, E>(tid, e)] = r[e];
+}
+
+// digits[j][m], m = 0 .. limbs (limbs: P), m != j: digit j of t2, centered, lifted to modulus m, through
+// the stages that couple the parts of its transform (below 8q). One thread per (j, m) and R coefficients.
+template <int LOGN>
+__global__ void __launch_bounds__(128) k_relin_digits(const __grid_constant__ SqImgArgs a, const u64* t2, u64* digits)
+{
+    constexpr int LS = kRelinLs<LOGN>, R = 1 << LS, M = 1 << (LOGN - LS);
     const int nm = a.limbs + 1;
-    const int jm = blockIdx.y;                 // j * nm + m
-    const int j = jm / nm, m = jm % nm;
-    const int mod = m < a.limbs ? m : a.L;     // index into the moduli (P at index L)
-    const u64 qj = a.rns.q[j], qm = a.rns.q[mod];
-    const u64 half = (qj - 1) / 2;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const u64 v = d2[(size_t)j * n + i];
-        u64 out;
-        if (v <= half) {
-            out = reduce64(v, qm, a.mu[mod]);
-        } else {
-            const u64 mag = reduce64(qj - v, qm, a.mu[mod]);
-            out = mag == 0 ? 0 : qm - mag;
-        }
-        digits[(size_t)jm * n + i] = out;
+    const int j = blockIdx.y / a.limbs, mj = blockIdx.y % a.limbs, m = mj + (mj >= j ? 1 : 0);
+    const int mod = m < a.limbs ? m : a.L;
+    const u64 qj = a.rns.q[j], q = a.rns.q[mod], mu = a.rns.mu[mod], half = (qj - 1) / 2;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= M) return;
+    u64 r[R];
+#pragma unroll
+    for (int k = 0; k < R; ++k) r[k] = t2[((size_t)j << LOGN) + k * M + i];
+    inv_tail<LS, 8>(r, a.rns.tab[j].itw, qj);
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+        const u64 v = below1<4>(r[k], qj), mag = reduce64(v <= half ? v : qj - v, q, mu);
+        r[k] = v <= half || mag == 0 ? mag : q - mag;
     }
+    fwd_head<LS, 8>(r, a.rns.tab[mod].tw, q);
+#pragma unroll
+    for (int k = 0; k < R; ++k) digits[((size_t)(j * nm + m) << LOGN) + k * M + i] = r[k];
 }
 
-cudaError_t launch_relin_digits(const RelinArgs& a, const u64* d2, u64* digits, cudaStream_t st)
+// The parts of the digits' transforms, in place (below 8q). Block ((j, m != j), part).
+template <int LOGN>
+__global__ void __launch_bounds__((1 << (LOGN - kRelinLs<LOGN>)) / 8) k_relin_fwd(const __grid_constant__ SqImgArgs a,
+                                                                                u64* digits)
 {
-    dim3 grid((1u << a.rns.logn) / 256, a.limbs * (a.limbs + 1));
-    k_relin_digits<<<grid, 256, 0, st>>>(a, d2, digits);
-    return cudaGetLastError();
-}
-
-__global__ void k_relin_mac(const __grid_constant__ RelinArgs a, const u64* digits_hat, u64* acc)
-{
-    const int n = 1 << a.rns.logn;
-    const int nm = a.limbs + 1;
-    const int bm = blockIdx.y;                 // b * nm + m
-    const int b = bm / nm, m = bm % nm;
+    constexpr int LS = kRelinLs<LOGN>, LOGM = LOGN - LS, E = 8, LAST = NttShape<LOGM, E>::LAST;
+    extern __shared__ u64 sm[];
+    const int tid = threadIdx.x, jm = blockIdx.x >> LS, h = blockIdx.x & ((1 << LS) - 1);
+    const int j = jm / a.limbs, mj = jm % a.limbs, m = mj + (mj >= j ? 1 : 0);
     const int mod = m < a.limbs ? m : a.L;
     const u64 q = a.rns.q[mod];
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        u64 s = 0;
-        for (int j = 0; j < a.limbs; ++j) {
-            const size_t ko = (((size_t)j * 2 + b) * (a.L + 1) + mod) * n + i;
-            const u64 d = digits_hat[((size_t)j * nm + m) * n + i];
-            s = add_mod(s, shoup(d, a.evk_hat[ko], a.evk_hat_p[ko], q), q);
+    u64* d = digits + ((size_t)(j * (a.limbs + 1) + m) << LOGN) + ((size_t)h << LOGM);
+    u64 r[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) r[e] = d[elem_index<LOGM, 0, E>(tid, e)];
+    ntt_fwd_regs<LOGM, false, E, 8, 8>(sm, r, tid, a.rns.tab[mod], q, (1 << LS) + h);
+#pragma unroll
+    for (int e = 0; e < E; ++e) d[elem_index<LOGM, LAST, E>(tid, e)] = r[e];
+}
+
+// acc[b][m] = the parts of INTT(sum_{j != m} digit_j^ evk_j^[b][m] + (P N^{-1} 2^64) t_b^ + t2^ 2^64 evk_m^[b][m])
+// (the last two for m < limbs), below 4q. Block ((b, m), part).
+template <int LOGN>
+__global__ void __launch_bounds__((1 << (LOGN - kRelinLs<LOGN>)) / 8)
+    k_relin_acc(const __grid_constant__ SqImgArgs a, const u64* tensor, const u64* digits, u64* acc)
+{
+    constexpr int LS = kRelinLs<LOGN>, LOGM = LOGN - LS, E = 8, LAST = NttShape<LOGM, E>::LAST;
+    extern __shared__ u64 sm[];
+    const int tid = threadIdx.x, bm = blockIdx.x >> LS, h = blockIdx.x & ((1 << LS) - 1);
+    const int nm = a.limbs + 1, b = bm / nm, m = bm % nm;
+    const int mod = m < a.limbs ? m : a.L;
+    const u64 q = a.rns.q[mod];
+    const size_t part = (size_t)h << LOGM;
+    u64 r[E];
+#pragma unroll
+    for (int e = 0; e < E; ++e) r[e] = 0;
+    for (int j = 0; j < a.limbs; ++j) {
+        const size_t key = ((((size_t)j * 2 + b) * (a.L + 1) + mod) << LOGN) + part;
+        const u64* d = (j == m ? tensor + ((size_t)(2 * a.limbs + m) << LOGN) : digits + ((size_t)(j * nm + m) << LOGN)) + part;
+#pragma unroll
+        for (int e = 0; e < E; ++e) {
+            const int x = elem_index<LOGM, LAST, E>(tid, e);
+            u64 v = d[x];
+            if (j == m) v = shoup3(v, a.r64[m], a.r64_p[m], q);
+            r[e] = halve<8>(r[e] + shoup3(v, __ldg(a.evk_hat + key + x), __ldg(a.evk_hat_p + key + x), q), q);
         }
-        acc[(size_t)bm * n + i] = s;
+    }
+    if (m < a.limbs) {
+        const u64* t = tensor + ((size_t)(b * a.limbs + m) << LOGN) + part;
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            r[e] = halve<8>(r[e] + shoup3(t[elem_index<LOGM, LAST, E>(tid, e)], a.pn[m], a.pn_p[m], q), q);
+    }
+    ntt_inv_regs<LOGM, false, E, 8>(sm, r, tid, a.rns.tab[mod], q, (1 << LS) + h);
+    u64* o = acc + ((size_t)bm << LOGN) + part;
+#pragma unroll
+    for (int e = 0; e < E; ++e) o[elem_index<LOGM, 0, E>(tid, e)] = r[e];
+}
+
+// out_b[j], j < t = limbs - 1: the last coupling stages of acc[b][P], acc[b][t] and acc[b][j], mod-down by P,
+// rescale by q_t. One thread per (b, j) and R coefficients.
+template <int LOGN>
+__global__ void __launch_bounds__(128) k_relin_out(const __grid_constant__ SqImgArgs a, const u64* acc)
+{
+    constexpr int LS = kRelinLs<LOGN>, R = 1 << LS, M = 1 << (LOGN - LS);
+    const int nm = a.limbs + 1, t = a.limbs - 1;
+    const int b = blockIdx.y / t, j = blockIdx.y % t;
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= M) return;
+    const u64 P = a.rns.q[a.L], halfP = (P - 1) / 2;
+    u64 ap[R], lt[R], r[R];
+    auto load = [&](int m, int mod, u64 (&v)[R]) {
+#pragma unroll
+        for (int k = 0; k < R; ++k) v[k] = acc[((size_t)(b * nm + m) << LOGN) + k * M + i];
+        inv_tail<LS, 8>(v, a.rns.tab[mod].itw, a.rns.q[mod]);
+    };
+    auto mod_down = [&](u64 v, u64 p, int m) {   // (v - [p]_centered) P^{-1} mod q_m, v below 4 q_m
+        const u64 q = a.rns.q[m];
+        u64 lp = reduce64(p, q, a.rns.mu[m]);
+        if (p > halfP) lp = add_mod(lp, a.neg_p_mod[m], q);
+        return shoup(v + q - lp, a.p_inv[m], a.p_inv_p[m], q);
+    };
+    load(a.limbs, a.L, ap);
+#pragma unroll
+    for (int k = 0; k < R; ++k) ap[k] = below1<4>(ap[k], P);
+    load(t, t, lt);
+    load(j, j, r);
+    const u64 q = a.rns.q[j];
+    u64* o = a.out + ((size_t)(b * t + j) << LOGN) + i;
+#pragma unroll
+    for (int k = 0; k < R; ++k) {
+        const u64 ct = mod_down(lt[k], ap[k], t), cj = mod_down(r[k], ap[k], j);
+        const u64 u = shoup_lazy(cj, a.qt_inv[j], a.qt_inv_p[j], q);
+        const u64 w = shoup_lazy(ct, a.qt_inv[j], a.qt_inv_p[j], q);
+        u64 v = csub_s(csub_s(u + 2 * q - w, 2 * q), q);
+        if (ct > a.half_qt) v = add_mod(v, 1, q);
+        o[k * M] = v;
     }
 }
 
-cudaError_t launch_relin_mac(const RelinArgs& a, const u64* digits_hat, u64* acc, cudaStream_t st)
+template <int LOGN>
+static cudaError_t relin_launch(const SqImgArgs& a, const u64* tensor, u64* t2, u64* digits, u64* acc, cudaStream_t st)
 {
-    dim3 grid((1u << a.rns.logn) / 256, 2 * (a.limbs + 1));
-    k_relin_mac<<<grid, 256, 0, st>>>(a, digits_hat, acc);
+    constexpr int LS = kRelinLs<LOGN>, R = 1 << LS, M = 1 << (LOGN - LS), T = M / 8;
+    const size_t smem = (size_t)M * 8;
+    const int limbs = a.limbs;
+    k_relin_t2<LOGN><<<limbs * R, T, smem, st>>>(a, tensor + ((size_t)2 * limbs << LOGN), t2);
+    k_relin_digits<LOGN><<<dim3((M + 127) / 128, limbs * limbs), 128, 0, st>>>(a, t2, digits);
+    k_relin_fwd<LOGN><<<limbs * limbs * R, T, smem, st>>>(a, digits);
+    k_relin_acc<LOGN><<<2 * (limbs + 1) * R, T, smem, st>>>(a, tensor, digits, acc);
+    k_relin_out<LOGN><<<dim3((M + 127) / 128, 2 * (limbs - 1)), 128, 0, st>>>(a, acc);
     return cudaGetLastError();
 }
 
-__global__ void k_relin_moddown(const __grid_constant__ RelinArgs a, const u64* d01, const u64* acc, u64* out)
+cudaError_t launch_relin_rescale(const SqImgArgs& a, const u64* tensor, u64* t2, u64* digits, u64* acc, cudaStream_t st)
 {
-    const int n = 1 << a.rns.logn;
-    const int nm = a.limbs + 1;
-    const int bj = blockIdx.y;                 // b * limbs + j
-    const int b = bj / a.limbs, j = bj % a.limbs;
-    const u64 qj = a.rns.q[j];
-    const u64 P = a.rns.q[a.L];
-    const u64 halfP = (P - 1) / 2;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-        const u64 ap = acc[((size_t)b * nm + a.limbs) * n + i];
-        u64 r = reduce64(ap, qj, a.mu[j]);
-        if (ap > halfP) r = add_mod(r, a.neg_p_mod[j], qj);   // (acc_P - P) mod q_j
-        const u64 aj = acc[((size_t)b * nm + j) * n + i];
-        const u64 ks = shoup(sub_mod(aj, r, qj), a.p_inv[j], a.p_inv_p[j], qj);
-        out[(size_t)bj * n + i] = add_mod(d01[(size_t)bj * n + i], ks, qj);
+    switch (a.rns.logn) {
+    case 10: return relin_launch<10>(a, tensor, t2, digits, acc, st);
+    case 11: return relin_launch<11>(a, tensor, t2, digits, acc, st);
+    case 12: return relin_launch<12>(a, tensor, t2, digits, acc, st);
+    case 13: return relin_launch<13>(a, tensor, t2, digits, acc, st);
+    case 14: return relin_launch<14>(a, tensor, t2, digits, acc, st);
+    default: return cudaErrorInvalidValue;
     }
-}
-
-cudaError_t launch_relin_moddown(const RelinArgs& a, const u64* d01, const u64* acc, u64* out, cudaStream_t st)
-{
-    dim3 grid((1u << a.rns.logn) / 256, 2 * a.limbs);
-    k_relin_moddown<<<grid, 256, 0, st>>>(a, d01, acc, out);
-    return cudaGetLastError();
 }
 
 }  // namespace ichee

@@ -264,9 +264,11 @@ __host__ __device__ constexpr int fwd_bound(int cap, int b, int S)
 }
 
 // Forward stages S0 .. S0+S-1 on registers below B q. Stage s pairs x with x + N/2^{s+1} and uses
-// twiddle index 2^s + (x >> (LOGN - s)).
+// twiddle index root 2^s + (x >> (LOGN - s)): root = 1 for a whole transform; for part h of the 2^r
+// equal parts that the first r stages of a longer transform leave, root = 2^r + h and the longer
+// transform's table.
 template <int LOGN, int S0, int E, bool WT, int CAP, int B>
-__device__ __forceinline__ void fwd_regs(u64 (&r)[E], int tid, const ulonglong2* __restrict__ tw, u64 q)
+__device__ __forceinline__ void fwd_regs(u64 (&r)[E], int tid, const ulonglong2* __restrict__ tw, u64 q, int root)
 {
     using P = Pass<LOGN, S0, E>;
     static_for<P::G>([&](auto gc) {
@@ -277,7 +279,7 @@ __device__ __forceinline__ void fwd_regs(u64 (&r)[E], int tid, const ulonglong2*
             constexpr bool fold = fwd_bound(CAP, B, k) + 4 > CAP;
             static_for<(1 << k)>([&](auto bc) {
                 constexpr int b = decltype(bc)::v;
-                const ulonglong2 w = __ldg(tw + (1 << s) + (h << k) + b);
+                const ulonglong2 w = __ldg(tw + (root << s) + (h << k) + b);
 #pragma unroll
                 for (int jj = b * 2 * half; jj < b * 2 * half + half; ++jj) {
                     const int i0 = g * (1 << P::S) + jj, i1 = i0 + half;
@@ -310,7 +312,7 @@ __host__ __device__ constexpr int inv_bound(int cap, int b, int S)
 
 // Inverse stages S0+S-1 .. S0 (reverse order) on registers below B q (B <= CAP/2).
 template <int LOGN, int S0, int E, bool WT, int CAP, int B>
-__device__ __forceinline__ void inv_regs(u64 (&r)[E], int tid, const ulonglong2* __restrict__ itw, u64 q)
+__device__ __forceinline__ void inv_regs(u64 (&r)[E], int tid, const ulonglong2* __restrict__ itw, u64 q, int root)
 {
     using P = Pass<LOGN, S0, E>;
     static_for<P::G>([&](auto gc) {
@@ -320,7 +322,7 @@ __device__ __forceinline__ void inv_regs(u64 (&r)[E], int tid, const ulonglong2*
             constexpr int t = decltype(tc)::v, k = P::S - 1 - t, s = S0 + k, half = 1 << t;
             static_for<(1 << k)>([&](auto bc) {
                 constexpr int b = decltype(bc)::v;
-                const ulonglong2 w = __ldg(itw + (1 << s) + (h << k) + b);
+                const ulonglong2 w = __ldg(itw + (root << s) + (h << k) + b);
                 static_for<half>([&](auto jc) {
                     constexpr int j0 = b * 2 * half + decltype(jc)::v;
                     constexpr int i0 = g * (1 << P::S) + j0, i1 = i0 + half;
@@ -337,31 +339,70 @@ __device__ __forceinline__ void inv_regs(u64 (&r)[E], int tid, const ulonglong2*
 // Forward passes after the first: on entry r holds the output of pass S0-LE (its layout), on
 // exit the output of the last pass in the last pass's layout.
 template <int LOGN, int S0, int E, int CAP, int B>
-__device__ __forceinline__ void fwd_rest(u64* sm, u64 (&r)[E], int tid, const ulonglong2* __restrict__ tw, u64 q)
+__device__ __forceinline__ void fwd_rest(u64* sm, u64 (&r)[E], int tid, const ulonglong2* __restrict__ tw, u64 q, int root)
 {
     constexpr int LE = Radix<E>::LE;
     if constexpr (S0 <= NttShape<LOGN, E>::LAST) {
         store_sm<LOGN, S0 - LE, E>(sm, r, tid);
         exchange_barrier<LOGN, S0, E>();
         load_sm<LOGN, S0, E>(sm, r, tid);
-        fwd_regs<LOGN, S0, E, true, CAP, B>(r, tid, tw, q);
-        fwd_rest<LOGN, S0 + LE, E, CAP, fwd_bound(CAP, B, Pass<LOGN, S0, E>::S)>(sm, r, tid, tw, q);
+        fwd_regs<LOGN, S0, E, true, CAP, B>(r, tid, tw, q, root);
+        fwd_rest<LOGN, S0 + LE, E, CAP, fwd_bound(CAP, B, Pass<LOGN, S0, E>::S)>(sm, r, tid, tw, q, root);
     }
 }
 
 // Inverse passes S0, S0-LE, ..., 0: on entry r holds bit-reversed data in the layout of pass
 // S0 (no inverse stage applied yet), on exit natural-order data in the layout of pass 0.
 template <int LOGN, int S0, int E, int CAP, int B>
-__device__ __forceinline__ void inv_rest(u64* sm, u64 (&r)[E], int tid, const ulonglong2* __restrict__ itw, u64 q)
+__device__ __forceinline__ void inv_rest(u64* sm, u64 (&r)[E], int tid, const ulonglong2* __restrict__ itw, u64 q, int root)
 {
     constexpr int LE = Radix<E>::LE;
-    inv_regs<LOGN, S0, E, true, CAP, B>(r, tid, itw, q);
+    inv_regs<LOGN, S0, E, true, CAP, B>(r, tid, itw, q, root);
     if constexpr (S0 > 0) {
         store_sm<LOGN, S0, E>(sm, r, tid);
         exchange_barrier<LOGN, S0, E>();
         load_sm<LOGN, S0 - LE, E>(sm, r, tid);
-        inv_rest<LOGN, S0 - LE, E, CAP, inv_bound(CAP, B, Pass<LOGN, S0, E>::S)>(sm, r, tid, itw, q);
+        inv_rest<LOGN, S0 - LE, E, CAP, inv_bound(CAP, B, Pass<LOGN, S0, E>::S)>(sm, r, tid, itw, q, root);
     }
+}
+
+// The first LS stages of a forward transform on the R = 2^LS coefficients i + j N/R of one i (r[j] below
+// q on entry, below fwd_bound(CAP, 1, LS) q on exit), and the last LS of an inverse one (below 4q on
+// entry, below CAP/2 q on exit): what couples the R parts of a transform split over blocks.
+template <int LS, int CAP>
+__device__ __forceinline__ void fwd_head(u64 (&r)[1 << LS], const ulonglong2* __restrict__ tw, u64 q)
+{
+    static_for<LS>([&](auto kc) {
+        constexpr int k = decltype(kc)::v, half = 1 << (LS - 1 - k);
+        constexpr bool fold = fwd_bound(CAP, 1, k) + 4 > CAP;
+#pragma unroll
+        for (int i = 0; i < 1 << LS; ++i) {
+            if (i & half) continue;
+            const ulonglong2 w = __ldg(tw + (1 << k) + i / (2 * half));
+            const u64 X = fold ? halve<CAP>(r[i], q) : r[i];
+            const u64 T = shoup3(r[i + half], w.x, w.y, q);
+            r[i] = X + T;
+            r[i + half] = X - T + 4 * q;
+        }
+    });
+}
+
+template <int LS, int CAP>
+__device__ __forceinline__ void inv_tail(u64 (&r)[1 << LS], const ulonglong2* __restrict__ itw, u64 q)
+{
+    static_for<LS>([&](auto tc) {
+        constexpr int t = decltype(tc)::v, k = LS - 1 - t, half = 1 << t;
+        static_for<(1 << LS)>([&](auto ic) {
+            constexpr int i = decltype(ic)::v;
+            if constexpr (!(i & half)) {
+                constexpr int bound = inv_before(CAP, 4, t, i);
+                const ulonglong2 w = __ldg(itw + (1 << k) + i / (2 * half));
+                const u64 X = r[i], Y = r[i + half];
+                r[i] = 2 * bound > CAP / 2 ? halve<CAP>(X + Y, q) : X + Y;
+                r[i + half] = shoup3(X - Y + bound * q, w.x, w.y, q);
+            }
+        });
+    });
 }
 
 // ---------------------------------------------------------------------------------------
@@ -480,12 +521,12 @@ template <int LOGN, bool COMPACT, int CAP, int B>
 __host__ __device__ constexpr int fwd_out() { return COMPACT ? CAP : fwd_bound(CAP, B, LOGN); }
 
 template <int LOGN, bool COMPACT, int E, int CAP, int B>
-__device__ __forceinline__ void ntt_fwd_regs(u64* sm, u64 (&r)[E], int tid, const ModTables& t, u64 q)
+__device__ __forceinline__ void ntt_fwd_regs(u64* sm, u64 (&r)[E], int tid, const ModTables& t, u64 q, int root = 1)
 {
     constexpr int LE = Radix<E>::LE;
     if constexpr (!COMPACT) {
-        fwd_regs<LOGN, 0, E, true, CAP, B>(r, tid, t.tw, q);
-        fwd_rest<LOGN, LE, E, CAP, fwd_bound(CAP, B, Pass<LOGN, 0, E>::S)>(sm, r, tid, t.tw, q);
+        fwd_regs<LOGN, 0, E, true, CAP, B>(r, tid, t.tw, q, root);
+        fwd_rest<LOGN, LE, E, CAP, fwd_bound(CAP, B, Pass<LOGN, 0, E>::S)>(sm, r, tid, t.tw, q, root);
         return;
     }
     constexpr int NFULL = LOGN / LE, TAIL = LOGN % LE;
@@ -505,23 +546,23 @@ __device__ __forceinline__ void ntt_fwd_regs(u64* sm, u64 (&r)[E], int tid, cons
         store_sm_rt<E>(sm, r, tid, LOGN - LE * NFULL);
         __syncthreads();
         load_sm<LOGN, LE * NFULL, E, false>(sm, r, tid);
-        fwd_regs<LOGN, LE * NFULL, E, false, CAP, CAP>(r, tid, t.tw, q);
+        fwd_regs<LOGN, LE * NFULL, E, false, CAP, CAP>(r, tid, t.tw, q, 1);
     }
 }
 
 // Whole inverse transform, input in registers in the layout of the last pass, below 4q; output in
 // registers in the layout of pass 0, natural order, below CAP/2 q.
 template <int LOGN, bool COMPACT, int E, int CAP>
-__device__ __forceinline__ void ntt_inv_regs(u64* sm, u64 (&r)[E], int tid, const ModTables& t, u64 q)
+__device__ __forceinline__ void ntt_inv_regs(u64* sm, u64 (&r)[E], int tid, const ModTables& t, u64 q, int root = 1)
 {
     constexpr int LE = Radix<E>::LE;
     if constexpr (!COMPACT) {
-        inv_rest<LOGN, NttShape<LOGN, E>::LAST, E, CAP, 4>(sm, r, tid, t.itw, q);
+        inv_rest<LOGN, NttShape<LOGN, E>::LAST, E, CAP, 4>(sm, r, tid, t.itw, q, root);
         return;
     }
     constexpr int NFULL = LOGN / LE, TAIL = LOGN % LE;
     if constexpr (TAIL > 0) {
-        inv_regs<LOGN, LE * NFULL, E, false, CAP, 4>(r, tid, t.itw, q);
+        inv_regs<LOGN, LE * NFULL, E, false, CAP, 4>(r, tid, t.itw, q, 1);
         store_sm<LOGN, LE * NFULL, E, false>(sm, r, tid);
         __syncthreads();
         load_sm_rt<E>(sm, r, tid, LOGN - LE * NFULL);

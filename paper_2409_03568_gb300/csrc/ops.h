@@ -93,7 +93,7 @@ cudaError_t launch_radix_meanfilter3_batch(const RadixArgs& ra, const OpsArgs& a
 // Matching: sum over ciphertexts of (a - b)^2 as a degree-2 ciphertext in the NTT domain.
 // At N = 2^14 the accumulation runs split: each polynomial as two 2^13-point halves after the
 // transform's first stage (sqdiff_split(logn)), block j taking limb j % limbs and half
-// (j / limbs) % 2, with twiddle tables per half (htab).
+// (j / limbs) % 2.
 __host__ __device__ inline bool sqdiff_split(int logn) { return logn == 14; }
 // Accumulating blocks an SM holds: 1024 threads' worth (2^13 / 8 threads a block at N = 2^13 and 2^14).
 __host__ __device__ constexpr int sqdiff_blocks_per_sm(int logn) { return logn >= 13 ? 1 : 1 << (13 - logn); }
@@ -105,7 +105,6 @@ struct SqDiffArgs {
     const u64* b;
     u64* partial;                  // [n_blocks][4][N] (split: [n_blocks][4][N/2]) scratch
     int n_blocks;                  // a multiple of limbs (split: of 2 limbs)
-    ModTables htab[2][kMaxPrimes]; // split: twiddles of the two half transforms
 };
 cudaError_t launch_sqdiff_accumulate(const SqDiffArgs& a, cudaStream_t st);
 // tensor[p][l][x] = (add ? tensor[p][l][x] mod q_l : 0) + the sum over the blocks of limb l (and,
@@ -115,18 +114,6 @@ cudaError_t launch_sqdiff_reduce(const RnsArgs& rns, int limbs, const u64* parti
 // out[r][x] = in[r][x] mod q_{r % limbs}, rows of N words, any 64-bit input
 cudaError_t launch_reduce_rows(const RnsArgs& rns, int rows, int limbs, const u64* in, u64* out, cudaStream_t st);
 
-// Key switching of a degree-2 ciphertext (hybrid, one digit per ciphertext prime, one special
-// prime P).
-struct RelinArgs {
-    RnsArgs rns;                   // moduli q_0..q_{L-1}, P at index L
-    int L;                         // limbs of the key (full chain)
-    int limbs;                     // limbs of the ciphertext (t + 1)
-    const u64* evk_hat;            // [L][2][L+1][N] NTT domain
-    const u64* evk_hat_p;          // Shoup companions
-    u64 p_inv[kMaxPrimes], p_inv_p[kMaxPrimes];  // P^{-1} mod q_j (Shoup)
-    u64 neg_p_mod[kMaxPrimes];     // (-P) mod q_j
-    u64 mu[kMaxModuli];
-};
 // Per-pixel squared difference with relinearisation and rescale (one output ciphertext per
 // input pair). Moduli: q_0..q_{limbs-1} of the ciphertexts, P at index L of rns.
 struct SqImgArgs {
@@ -152,11 +139,10 @@ size_t sqdiff_image_scratch_words(int logn, int limbs);
 int sqdiff_image_grid(int logn, u64 n_ct, int num_sms);
 cudaError_t launch_sqdiff_image(const SqImgArgs& a, int grid, cudaStream_t st);
 
-// digits[j][m][N] = centered residue of d2 limb j lifted to modulus m (m = 0..limbs-1, then P)
-cudaError_t launch_relin_digits(const RelinArgs& a, const u64* d2, u64* digits, cudaStream_t st);
-// acc[b][m][N] = sum_j digits^[j][m] * evk^_j[b][m]
-cudaError_t launch_relin_mac(const RelinArgs& a, const u64* digits_hat, u64* acc, cudaStream_t st);
-// out_b[j] = d_b[j] + (acc_b[j] - [acc_b[P]]_centered) * P^{-1} mod q_j
-cudaError_t launch_relin_moddown(const RelinArgs& a, const u64* d01, const u64* acc, u64* out, cudaStream_t st);
+// Relinearisation and rescale of a degree-2 ciphertext tensor[3][limbs][N] in the transform domain
+// (residues below each prime, with the Montgomery factor 2^{-64}) into a.out (one ciphertext of
+// limbs - 1 limbs); a's keys and constants, not its inputs. Working memory: t2 [limbs][N], digits
+// [limbs][limbs + 1][N], acc [2][limbs + 1][N].
+cudaError_t launch_relin_rescale(const SqImgArgs& a, const u64* tensor, u64* t2, u64* digits, u64* acc, cudaStream_t st);
 
 }  // namespace ichee

@@ -78,10 +78,8 @@ template <int E> static int check(int logn)
 int main()
 {
     int bad = 0;
-    for (int logn = 10; logn <= 14; ++logn) {
-        if (logn <= 13) bad += check<8>(logn);
-        bad += check<16>(logn);
-    }
+    for (int logn = 8; logn <= 13; ++logn) bad += check<8>(logn);   // from 8: the parts of relinearisation's transforms
+    for (int logn = 10; logn <= 14; ++logn) bad += check<16>(logn);
     printf("bad %d\n", bad);
     return bad != 0;
 }

@@ -71,6 +71,14 @@ int main()
             bad += check_bounds<8>(logn, cap, 2) + check_bounds<16>(logn, cap, 2) + check_bounds<8>(logn, cap, 1);
             if (cap == 16) bad += check_bounds<8>(logn, cap, 6);
         }
+    // relinearisation's transforms in parts: 2 or 3 coupling stages from canonical values, then a part
+    for (int logm = 8; logm <= 11; ++logm) bad += check_bounds<8>(logm, 8, 8);
+    for (int ls = 2; ls <= 3; ++ls) {
+        if (fwd_bound(8, 1, ls) > 8 || inv_bound(8, 4, ls) > 4) ++bad;
+        for (int t = 0; t < ls; ++t)
+            for (int i = 0; i < (1 << ls); ++i)
+                if (2 * inv_before(8, 4, t, i) > 8) ++bad;
+    }
     if (fwd_bound(kNoFold, 6, 13) > 62 || fwd_bound(kNoFold, 2, 13) > 62) ++bad;
     printf("bad %d\n", bad);
     return bad != 0;
