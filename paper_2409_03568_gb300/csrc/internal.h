@@ -46,6 +46,8 @@ struct EncArgs {
     CdtTable cdt;
     u64* out;                  // [n_ct][2][L][N]
     int num_sms;               // persistent grid of the single-image kernel
+    int groups;                // few ciphertexts: the blocks that share one by limbs, and a bit for each
+    u32 third;                 // with limbs of three primes; both set at the launch
     const u32* idx;            // optional: encrypt only pixels idx[0 .. *n_idx) (device list)
     const u32* n_idx;
 };

@@ -362,8 +362,9 @@ __device__ __forceinline__ u64 enc_crt(const EncLimb& lm, u32 y0, u32 y1, u32 y2
     return csub_s(csub_s(lo, 2 * lm.q), lm.q);
 }
 
-template <int LOGN>
-__device__ __forceinline__ void encrypt_ct(const EncArgs& a, int p, u64 seed, u64 id, u64* ct, u64* smem)
+// The block's share of a ciphertext: all limbs or, with SPLIT, limbs group, group + groups, ...
+template <int LOGN, bool SPLIT>
+__device__ __forceinline__ void encrypt_ct(const EncArgs& a, int group, int p, u64 seed, u64 id, u64* ct, u64* smem)
 {
     using S = EncShape<LOGN>;
     constexpr int N = 1 << LOGN, E = S::E, T = S::T, NP = S::NP, LAST = NttShape<LOGN, E>::LAST;
@@ -402,8 +403,10 @@ __device__ __forceinline__ void encrypt_ct(const EncArgs& a, int p, u64 seed, u6
     // (each thread's coefficients of the ciphertext, which it overwrites with the residues below),
     // so that at most two primes' digits are in registers. Then the first two primes of every limb.
     int turn = 0;
+    const int first = SPLIT ? group : 0, step = SPLIT ? a.groups : 1;
 #pragma unroll 1
     for (int phase = a.aux.n == 3 ? 0 : 1; phase < 2; ++phase) {
+        if (SPLIT && phase == 0 && !((a.third >> group) & 1u)) continue;
         const int i0 = phase == 0 ? 2 : 0, i1 = phase == 0 ? 3 : 2;
 #pragma unroll 1
         for (int i = i0; i < i1; ++i) {
@@ -417,7 +420,7 @@ __device__ __forceinline__ void encrypt_ct(const EncArgs& a, int p, u64 seed, u6
             for (int e = 0; e < E; ++e) vh[(i - i0) * N + e * T + tid] = r[0][e];
         }
 #pragma unroll 1
-        for (int l = 0; l < L; ++l) {
+        for (int l = first; l < L; l += step) {
             const EncLimb& lm = a.limb[l];
             if (i0 >= lm.np) continue;
 #pragma unroll 1
@@ -489,7 +492,7 @@ __device__ __forceinline__ void encrypt_setup(const EncArgs& a, u64* smem)
     __syncthreads();
 }
 
-template <int LOGN>
+template <int LOGN, bool SPLIT>
 __global__ void __launch_bounds__(EncShape<LOGN>::T, EncShape<LOGN>::BLOCKS)
     k_encrypt_fresh(const __grid_constant__ EncArgs a)
 {
@@ -499,11 +502,12 @@ __global__ void __launch_bounds__(EncShape<LOGN>::T, EncShape<LOGN>::BLOCKS)
     // all pixels, or a listed subset (the misses of a value cache) shared evenly; one call site,
     // so the kernel holds one copy of the transform code
     const u64 n = a.idx != nullptr ? (u64)*a.n_idx : a.n_ct;
-    for (u64 g = blockIdx.x; g < n; g += gridDim.x) {
+    for (u64 u = blockIdx.x; u < (SPLIT ? n * a.groups : n); u += gridDim.x) {
+        const u64 g = SPLIT ? u / a.groups : u;
         const u64 k = a.idx != nullptr ? (u64)a.idx[g] : g;
         const int p = a.pixels[k];
         if (a.skip_lut != nullptr && a.skip_lut[p] >= 0) continue;  // uniform across the block
-        encrypt_ct<LOGN>(a, p, a.seed, a.id_base + k, a.out + k * ct_len, smem);
+        encrypt_ct<LOGN, SPLIT>(a, SPLIT ? (int)(u % a.groups) : 0, p, a.seed, a.id_base + k, a.out + k * ct_len, smem);
     }
 }
 
@@ -520,7 +524,7 @@ __global__ void __launch_bounds__(EncShape<LOGN>::T, EncShape<LOGN>::BLOCKS)
         const u64 k = g - t.start[s];
         const int p = t.px[s][k];
         if (a.skip_lut != nullptr && a.skip_lut[p] >= 0) continue;
-        encrypt_ct<LOGN>(a, p, t.seed[s], k, t.out[s] + k * ct_len, smem);
+        encrypt_ct<LOGN, false>(a, 0, p, t.seed[s], k, t.out[s] + k * ct_len, smem);
     }
 }
 
@@ -528,30 +532,51 @@ __global__ void __launch_bounds__(EncShape<LOGN>::T, EncShape<LOGN>::BLOCKS)
 // ciphertexts. With pixels to skip in-kernel the shares would be uneven, so there more blocks than
 // fit are launched.
 template <int LOGN>
-static unsigned enc_grid(u64 n, int num_sms, bool skips)
+static unsigned enc_grid(const EncArgs& a, u64 n, int num_sms)
 {
-    const u64 cap = (u64)num_sms * EncShape<LOGN>::BLOCKS * (skips ? 16 : 1);
+    const u64 cap = (u64)num_sms * EncShape<LOGN>::BLOCKS * (a.skip_lut != nullptr ? 16 : 1);
     return (unsigned)(n < cap ? n : cap);
 }
 
-template <int LOGN>
-static cudaError_t enc_launch(const EncArgs& a, cudaStream_t st)
+template <int LOGN, bool SPLIT>
+static cudaError_t enc_launch_as(const EncArgs& a, u64 n, cudaStream_t st)
 {
     using S = EncShape<LOGN>;
-    cudaError_t e = cudaFuncSetAttribute(k_encrypt_fresh<LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)S::SMEM);
+    cudaError_t e = cudaFuncSetAttribute(k_encrypt_fresh<LOGN, SPLIT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)S::SMEM);
     if (e != cudaSuccess) return e;
-    k_encrypt_fresh<LOGN><<<enc_grid<LOGN>(a.n_ct, a.num_sms, a.skip_lut != nullptr), S::T, S::SMEM, st>>>(a);
+    k_encrypt_fresh<LOGN, SPLIT><<<enc_grid<LOGN>(a, n, a.num_sms), S::T, S::SMEM, st>>>(a);
     return cudaGetLastError();
 }
 
+// Fewer than half as many ciphertexts as SMs (a cache's tables, a thumbnail): the limbs of each are
+// shared out over blocks, as long as every block has an SM to itself. Each block draws the samples and
+// transforms v again, but the limbs, most of the work, run side by side.
+// Measured, 3 limbs at N = 2^13: 38 ciphertexts 96.8 -> 51.8 us, 64 in two groups 96.9 -> 78.5; 5 limbs
+// at 2^14: 290 -> 113 and 204; 2 limbs at 2^10: 19.0 -> 14.7. With two blocks to an SM it gains little
+// or loses (4 limbs at 2^10, 304 ciphertexts: 35.4 -> 45.9; 3 at 2^12, 110: 53.7 -> 74.2), so the line
+// is one block to an SM. A kernel of its own: run-time groups in the general one cost it 1 %.
 template <int LOGN>
-static cudaError_t enc_batch_launch(const EncArgs& a, const SegTable& t, int num_sms, cudaStream_t st)
+static cudaError_t enc_launch(EncArgs a, cudaStream_t st)
+{
+    const u64 fit = (u64)a.num_sms / a.n_ct;
+    a.groups = fit < (u64)a.L ? (int)fit : a.L;
+    if (a.groups < 2) return enc_launch_as<LOGN, false>(a, a.n_ct, st);
+    a.third = 0;
+    for (int l = 0; l < a.L; ++l)
+        if (a.limb[l].np == 3) a.third |= 1u << (l % a.groups);
+    return enc_launch_as<LOGN, true>(a, a.n_ct * a.groups, st);
+}
+
+template <int LOGN>
+static cudaError_t enc_batch_launch(EncArgs a, const SegTable& t, int num_sms, cudaStream_t st)
 {
     using S = EncShape<LOGN>;
     cudaError_t e = cudaFuncSetAttribute(k_encrypt_fresh_batch<LOGN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          (int)S::SMEM);
     if (e != cudaSuccess) return e;
-    k_encrypt_fresh_batch<LOGN><<<enc_grid<LOGN>(t.start[t.n], num_sms, a.skip_lut != nullptr), S::T, S::SMEM, st>>>(a, t);
+    const unsigned grid = enc_grid<LOGN>(a, t.start[t.n], num_sms);
+    k_encrypt_fresh_batch<LOGN><<<grid, S::T, S::SMEM, st>>>(a, t);
     return cudaGetLastError();
 }
 

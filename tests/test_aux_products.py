@@ -150,3 +150,24 @@ def test_fresh_against_the_oracle(ring):
     ref = o.encrypt_pixels(px[3:], 78)
     assert np.array_equal(dst[1].cpu().numpy().view(np.uint64).reshape(2, 2, ctx.L, ctx.n), ref)
     ctx.close()
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("ring", [
+    dict(log_n=10, prime_bits=[30, 30], log2_scale=25),                # one and two groups
+    dict(log_n=11, prime_bits=[30, 60, 44, 45, 29], log2_scale=25),    # groups with and without three primes
+    dict(log_n=14, prime_bits=[60, 40, 40], log2_scale=30),
+], ids=lambda r: "n%d" % (1 << r["log_n"]))
+def test_few_ciphertexts_shared_out_by_limbs(ring):
+    """A call of so few pixels that several blocks share a ciphertext gives the first ciphertexts of a
+    larger call, for every number of groups and at both sides of each line."""
+    torch = pytest.importorskip("torch")
+    from paper_2409_03568_gb300 import ichee
+    ctx = ichee.Context(**ring)
+    ctx.keygen(8)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    px = torch.randint(0, 256, (sms,), dtype=torch.uint8, device="cuda")
+    whole, _ = ctx.encrypt(px, 1, sms, 1, 5)
+    for n in sorted({1} | {sms // g + d for g in range(2, ctx.L + 1) for d in (0, 1)}):
+        part, _ = ctx.encrypt(px[:n].clone(), 1, n, 1, 5)
+        assert torch.equal(part.view(torch.int64).flatten(), whole.view(torch.int64).flatten()[:part.numel()]), n
