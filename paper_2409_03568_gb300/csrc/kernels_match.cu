@@ -24,21 +24,43 @@ __device__ __forceinline__ void tensor_pair(u64* acc, int n, u64 d1x, u64 d1y, u
     add(acc + 2 * n, mont_lazy(d1x, d1x, q, qinv), mont_lazy(d1y, d1y, q, qinv));
 }
 
+// A transform's output (below B q) as the products take it: below 4q, or any of a modulus below 2^50.
+template <int B>
+__device__ __forceinline__ u64 for_products(u64 x, u64 q)
+{
+    if constexpr (B > 16) return x;
+    else return below4<B>(x, q);
+}
+
+// The tensor terms of all positions of a thread (last-pass layout) from the transforms of d0 (r[0]) and
+// d1 (r[1]), below B q.
+template <int LOGN, int E, int B>
+__device__ __forceinline__ void tensor_terms(u64* acc, const u64 (&r)[2][E], int tid, u64 q, u64 qinv)
+{
+#pragma unroll
+    for (int e = 0; e < E; e += 2)
+        tensor_pair(acc + elem_index<LOGN, NttShape<LOGN, E>::LAST, E>(tid, e), 1 << LOGN, for_products<B>(r[1][e], q),
+                    for_products<B>(r[1][e + 1], q), for_products<B>(r[0][e], q), for_products<B>(r[0][e + 1], q), q,
+                    qinv);
+}
+
 // One block per SM-sized share of the work: block j owns limb l = j % limbs and every
 // (n_blocks/limbs)-th ciphertext. Per ciphertext it forms d = a - b for its limb, transforms
 // d0 and d1, and accumulates (d0^2, d0 d1, d1^2) position by position into its own slice of
 // the scratch buffer (each position is owned by one thread, so no atomics are needed; the middle
-// term is doubled when the slices are added up). d0 is transformed and waits in one shared-memory
-// buffer, d1 in the other. Every thread parks and reads back only the slots of its own last-pass
-// registers -- the slots it loaded in the transform's last exchange -- so no barrier follows the
-// transform. Values stay lazily reduced throughout (ntt.cuh): the difference in [0, 2q), the
+// term is doubled when the slices are added up). From N = 2^12 a thread holds its 8 residues of both
+// polynomials in registers: they share the twiddle loads and the exchange barriers, give every warp two
+// independent chains, and reach the tensor terms without a detour through shared memory. Below, d0 is
+// transformed first and waits in its own slots of the second buffer: with many small blocks on an SM
+// that is as fast or faster (900 pairs at N = 2^10 139 us, both at once 147; 3600 at 2^11 487 and 489).
+// Values stay lazily reduced throughout (ntt.cuh): the difference in [0, 2q), the
 // transforms' outputs below 4q as the Montgomery products take them, the accumulators in [0, 2q).
 // Moduli below 2^50 (NOFOLD) need no reduction inside a transform at all.
-// Whole matching calls against the earlier form (a conditional subtraction per butterfly, exact
-// quotients, canonical values, one block of 16 residues a thread per SM below N = 2^13): 4096 pairs
-// at N = 2^13 with primes 60/40/60 2.59 -> 2.31 ms, 3072 pairs at N = 2^14 and five limbs 6.99 -> 6.60
-// ms, 1600 pairs at N = 2^12 0.74 -> 0.55 ms. The multiply pipe is about half busy: transforms,
-// exchanges and twiddle loads of the one block per SM follow each other between its barriers.
+// Whole matching calls, 4096 pairs at N = 2^13 with primes 60/40/60: 2.59 ms with a conditional
+// subtraction per butterfly, exact quotients and canonical values, 2.31 lazily reduced, 2.23 with the
+// exchange barriers of ntt.cuh, 2.13 with both polynomials at once; 1600 pairs at N = 2^12 0.74, 0.55,
+// 0.52 and 0.50. What bounds it: the multiply pipe, three quarters busy; the rest of the time goes
+// to exchanges and to the tensor terms' accumulators (in L2).
 template <int LOGN, int E, int CAP>
 __device__ __forceinline__ void sqdiff_accumulate(const SqDiffArgs& a, u64* buf)
 {
@@ -46,7 +68,6 @@ __device__ __forceinline__ void sqdiff_accumulate(const SqDiffArgs& a, u64* buf)
     constexpr int LAST = NttShape<LOGN, E>::LAST;
     constexpr int OUT = fwd_out<LOGN, false, CAP, 2>();
     u64* acc = a.partial + (size_t)blockIdx.x * 4 * N;
-    u64* d0buf = buf + N;
     const int tid = threadIdx.x;
     const int limbs = a.limbs;
     const int l = blockIdx.x % limbs;
@@ -67,32 +88,52 @@ __device__ __forceinline__ void sqdiff_accumulate(const SqDiffArgs& a, u64* buf)
     for (u64 k = start; k < a.n_ct; k += stride) {
         const u64* A = a.a + k * 2 * (u64)limbs * N;
         const u64* B = a.b + k * 2 * (u64)limbs * N;
-#pragma unroll 1
-        for (int pb = 0; pb < 2; ++pb) {
-            const int x0 = elem_index<LOGN, 0, E>(tid, 0);   // first-pass layout: x0 + elem_offset(e)
-            const u64* pa = A + ((u64)pb * limbs + l) * N + x0;
-            const u64* pbb = B + ((u64)pb * limbs + l) * N + x0;
-            u64 r[E];
+        const int x0 = elem_index<LOGN, 0, E>(tid, 0);   // first-pass layout: x0 + elem_offset(e)
+        if constexpr (LOGN >= 12) {
+            u64 r[2][E];
 #pragma unroll
-            for (int e = 0; e < E; ++e) {
-                const int x = elem_offset<LOGN, 0, E>(e);
-                r[e] = __ldcs(pa + x) + q - __ldcs(pbb + x);
+            for (int p = 0; p < 2; ++p) {
+                const u64* pa = A + ((u64)p * limbs + l) * N + x0;
+                const u64* pb = B + ((u64)p * limbs + l) * N + x0;
+#pragma unroll
+                for (int e = 0; e < E; ++e) {
+                    const int x = elem_offset<LOGN, 0, E>(e);
+                    r[p][e] = __ldcs(pa + x) + q - __ldcs(pb + x);
+                }
             }
-            // d0 is transformed in its parking buffer and d1 in the other one: d1's transform then
-            // starts after d0's block-wide exchanges, which every thread reaches only after its
-            // reads of the previous pixel, so it needs no barrier of its own
-            if (pb == 0) __syncthreads();
-            u64* dst = pb == 0 ? d0buf : buf;
-            ntt_fwd_regs<LOGN, false, E, CAP, 2>(dst, r, tid, t, q);
-            const int sb = slot_base<LOGN, LAST, E>(tid);
+            __syncthreads();   // the last exchange's loads of the previous pixel are over
+            ntt_fwd_polys<LOGN, E, CAP, 2>(buf, r, tid, t, q);
+            tensor_terms<LOGN, E, OUT>(acc, r, tid, q, qinv);
+        } else {
+            u64* d0buf = buf + N;
+#pragma unroll 1
+            for (int p = 0; p < 2; ++p) {
+                const u64* pa = A + ((u64)p * limbs + l) * N + x0;
+                const u64* pb = B + ((u64)p * limbs + l) * N + x0;
+                u64 r[E];
 #pragma unroll
-            for (int e = 0; e < E; ++e)
-                dst[slot_of<LOGN, LAST, E>(sb, e)] = CAP == kNoFold ? r[e] : below4<CAP == kNoFold ? 1 : OUT>(r[e], q);
-        }
-#pragma unroll   // unrolled: 2.62 -> 2.60 ms (the split kernel below keeps its loop: 2.45 -> 2.71 ms unrolled)
-        for (int e = 0; e < E; e += 2) {
-            const int x = elem_index<LOGN, LAST, E>(tid, e);
-            tensor_pair(acc + x, N, buf[swz<E>(x)], buf[swz<E>(x + 1)], d0buf[swz<E>(x)], d0buf[swz<E>(x + 1)], q, qinv);
+                for (int e = 0; e < E; ++e) {
+                    const int x = elem_offset<LOGN, 0, E>(e);
+                    r[e] = __ldcs(pa + x) + q - __ldcs(pb + x);
+                }
+                // d0 is transformed in its parking buffer and d1 in the other one: d1's transform then
+                // starts after d0's block-wide exchanges, which every thread reaches only after its
+                // reads of the previous pixel, so it needs no barrier of its own. Every thread parks
+                // and reads back only the slots of its own last-pass registers -- the slots it loaded
+                // in the transform's last exchange -- so no barrier follows the transform.
+                if (p == 0) __syncthreads();
+                u64* dst = p == 0 ? d0buf : buf;
+                ntt_fwd_regs<LOGN, false, E, CAP, 2>(dst, r, tid, t, q);
+                const int sb = slot_base<LOGN, LAST, E>(tid);
+#pragma unroll
+                for (int e = 0; e < E; ++e) dst[slot_of<LOGN, LAST, E>(sb, e)] = for_products<OUT>(r[e], q);
+            }
+#pragma unroll
+            for (int e = 0; e < E; e += 2) {
+                const int x = elem_index<LOGN, LAST, E>(tid, e);
+                tensor_pair(acc + x, N, buf[swz<E>(x)], buf[swz<E>(x + 1)], d0buf[swz<E>(x)], d0buf[swz<E>(x + 1)], q,
+                            qinv);
+            }
         }
     }
 }
@@ -110,16 +151,17 @@ __global__ void __launch_bounds__(NttShape<LOGN, E>::T, sqdiff_blocks_per_sm(LOG
 // takes limb j % limbs and half h = (j / limbs) % 2: it loads both halves of d = a - b, applies
 // the first-stage butterfly for its half only (the product W d_hi is made by both halves'
 // blocks: 1/14 more products), and runs the other 13 stages with the 2^13-point code -- 8
-// residues per thread, 1024 threads, no spills -- from root 2 + h of the table. Its tensor terms go to
-// a [4][N/2] slice. The two blocks of a half pair read the same ciphertexts at about the same time (one HBM read, one
-// L2 hit).
+// residues of both polynomials per thread, 1024 threads -- from root 2 + h of the table. Its tensor terms
+// go to a [4][N/2] slice. The two blocks of a half pair read the same ciphertexts at about the same
+// time (one HBM read, one L2 hit). 992 pairs of five limbs: 2.14 ms with the polynomials in turn, 2.08
+// with both at once (2.21 while the slot and twiddle addresses of every pass were kept, spilled, across
+// pixels: the opaque thread number below makes them anew).
 template <int CAP>
 __device__ __forceinline__ void sqdiff_accumulate_split(const SqDiffArgs& a, u64* buf)
 {
     constexpr int LOGH = 13, NH = 1 << LOGH, N = 2 * NH, E = 8;
     constexpr int LAST = NttShape<LOGH, E>::LAST;
     constexpr int IN = 6, OUT = fwd_out<LOGH, false, CAP, IN>();
-    u64* d0buf = buf + NH;
     const int tid = threadIdx.x;
     const int limbs = a.limbs;
     const int l = blockIdx.x % limbs;
@@ -141,32 +183,25 @@ __device__ __forceinline__ void sqdiff_accumulate_split(const SqDiffArgs& a, u64
     for (u64 k = start; k < a.n_ct; k += stride) {
         const u64* A = a.a + k * 2 * (u64)limbs * N;
         const u64* B = a.b + k * 2 * (u64)limbs * N;
-#pragma unroll 1
-        for (int pb = 0; pb < 2; ++pb) {
-            const int x0 = elem_index<LOGH, 0, E>(tid, 0);
-            const u64* pa = A + ((u64)pb * limbs + l) * N + x0;
-            const u64* pbb = B + ((u64)pb * limbs + l) * N + x0;
-            u64 r[E];
+        int tid = threadIdx.x;
+        asm volatile("" : "+r"(tid));
+        const int x0 = elem_index<LOGH, 0, E>(tid, 0);
+        u64 r[2][E];
+#pragma unroll
+        for (int p = 0; p < 2; ++p) {
+            const u64* pa = A + ((u64)p * limbs + l) * N + x0;
+            const u64* pb = B + ((u64)p * limbs + l) * N + x0;
 #pragma unroll
             for (int e = 0; e < E; ++e) {
                 const int x = elem_offset<LOGH, 0, E>(e);
-                const u64 lo = pa[x] + q - pbb[x];                          // [0, 2q)
-                const u64 tt = shoup3(pa[x + NH] + q - pbb[x + NH], w1.x, w1.y, q);   // [0, 4q)
-                r[e] = h ? lo + 4 * q - tt : lo + tt;                       // below IN q
+                const u64 lo = pa[x] + q - pb[x];                                   // [0, 2q)
+                const u64 tt = shoup3(pa[x + NH] + q - pb[x + NH], w1.x, w1.y, q);   // [0, 4q)
+                r[p][e] = h ? lo + 4 * q - tt : lo + tt;                            // below IN q
             }
-            if (pb == 0) __syncthreads();   // d0 in its parking buffer, d1 in the other (as above)
-            u64* dst = pb == 0 ? d0buf : buf;
-            ntt_fwd_regs<LOGH, false, E, CAP, IN>(dst, r, tid, t, q, 2 + h);
-            const int sb = slot_base<LOGH, LAST, E>(tid);
-#pragma unroll
-            for (int e = 0; e < E; ++e)
-                dst[slot_of<LOGH, LAST, E>(sb, e)] = CAP == kNoFold ? r[e] : below4<CAP == kNoFold ? 1 : OUT>(r[e], q);
         }
-#pragma unroll 1
-        for (int e = 0; e < E; e += 2) {
-            const int x = elem_index<LOGH, LAST, E>(tid, e);
-            tensor_pair(acc + x, NH, buf[swz<E>(x)], buf[swz<E>(x + 1)], d0buf[swz<E>(x)], d0buf[swz<E>(x + 1)], q, qinv);
-        }
+        __syncthreads();   // the last exchange's loads of the previous pixel are over
+        ntt_fwd_polys<LOGH, E, CAP, IN>(buf, r, tid, t, q, 2 + h);
+        tensor_terms<LOGH, E, OUT>(acc, r, tid, q, qinv);
     }
 }
 

@@ -267,8 +267,8 @@ __host__ __device__ constexpr int fwd_bound(int cap, int b, int S)
 // twiddle index root 2^s + (x >> (LOGN - s)): root = 1 for a whole transform; for part h of the 2^r
 // equal parts that the first r stages of a longer transform leave, root = 2^r + h and the longer
 // transform's table.
-template <int LOGN, int S0, int E, bool WT, int CAP, int B>
-__device__ __forceinline__ void fwd_regs(u64 (&r)[E], int tid, const ulonglong2* __restrict__ tw, u64 q, int root)
+template <int LOGN, int S0, int E, bool WT, int CAP, int B, int NP>
+__device__ __forceinline__ void fwd_regs(u64 (&r)[NP][E], int tid, const ulonglong2* __restrict__ tw, u64 q, int root)
 {
     using P = Pass<LOGN, S0, E>;
     static_for<P::G>([&](auto gc) {
@@ -282,11 +282,14 @@ __device__ __forceinline__ void fwd_regs(u64 (&r)[E], int tid, const ulonglong2*
                 const ulonglong2 w = __ldg(tw + (root << s) + (h << k) + b);
 #pragma unroll
                 for (int jj = b * 2 * half; jj < b * 2 * half + half; ++jj) {
-                    const int i0 = g * (1 << P::S) + jj, i1 = i0 + half;
-                    const u64 X = fold ? halve<CAP>(r[i0], q) : r[i0];
-                    const u64 T = shoup3(r[i1], w.x, w.y, q);
-                    r[i0] = X + T;
-                    r[i1] = X - T + 4 * q;
+#pragma unroll
+                    for (int p = 0; p < NP; ++p) {
+                        const int i0 = g * (1 << P::S) + jj, i1 = i0 + half;
+                        const u64 X = fold ? halve<CAP>(r[p][i0], q) : r[p][i0];
+                        const u64 T = shoup3(r[p][i1], w.x, w.y, q);
+                        r[p][i0] = X + T;
+                        r[p][i1] = X - T + 4 * q;
+                    }
                 }
             });
         });
@@ -337,18 +340,30 @@ __device__ __forceinline__ void inv_regs(u64 (&r)[E], int tid, const ulonglong2*
 }
 
 // Forward passes after the first: on entry r holds the output of pass S0-LE (its layout), on
-// exit the output of the last pass in the last pass's layout.
-template <int LOGN, int S0, int E, int CAP, int B>
-__device__ __forceinline__ void fwd_rest(u64* sm, u64 (&r)[E], int tid, const ulonglong2* __restrict__ tw, u64 q, int root)
+// exit the output of the last pass in the last pass's layout. Polynomial p exchanges through
+// sm + p N; the polynomials share the barriers.
+template <int LOGN, int S0, int E, int CAP, int B, int NP>
+__device__ __forceinline__ void fwd_rest(u64* sm, u64 (&r)[NP][E], int tid, const ulonglong2* __restrict__ tw, u64 q, int root)
 {
     constexpr int LE = Radix<E>::LE;
     if constexpr (S0 <= NttShape<LOGN, E>::LAST) {
-        store_sm<LOGN, S0 - LE, E>(sm, r, tid);
+#pragma unroll
+        for (int p = 0; p < NP; ++p) store_sm<LOGN, S0 - LE, E>(sm + (p << LOGN), r[p], tid);
         exchange_barrier<LOGN, S0, E>();
-        load_sm<LOGN, S0, E>(sm, r, tid);
+#pragma unroll
+        for (int p = 0; p < NP; ++p) load_sm<LOGN, S0, E>(sm + (p << LOGN), r[p], tid);
         fwd_regs<LOGN, S0, E, true, CAP, B>(r, tid, tw, q, root);
         fwd_rest<LOGN, S0 + LE, E, CAP, fwd_bound(CAP, B, Pass<LOGN, S0, E>::S)>(sm, r, tid, tw, q, root);
     }
+}
+
+// NP whole forward transforms, every pass unrolled.
+template <int LOGN, int E, int CAP, int B, int NP>
+__device__ __forceinline__ void ntt_fwd_polys(u64* sm, u64 (&r)[NP][E], int tid, const ModTables& t, u64 q, int root = 1)
+{
+    constexpr int LE = Radix<E>::LE;
+    fwd_regs<LOGN, 0, E, true, CAP, B>(r, tid, t.tw, q, root);
+    fwd_rest<LOGN, LE, E, CAP, fwd_bound(CAP, B, Pass<LOGN, 0, E>::S)>(sm, r, tid, t.tw, q, root);
 }
 
 // Inverse passes S0, S0-LE, ..., 0: on entry r holds bit-reversed data in the layout of pass
@@ -525,8 +540,7 @@ __device__ __forceinline__ void ntt_fwd_regs(u64* sm, u64 (&r)[E], int tid, cons
 {
     constexpr int LE = Radix<E>::LE;
     if constexpr (!COMPACT) {
-        fwd_regs<LOGN, 0, E, true, CAP, B>(r, tid, t.tw, q, root);
-        fwd_rest<LOGN, LE, E, CAP, fwd_bound(CAP, B, Pass<LOGN, 0, E>::S)>(sm, r, tid, t.tw, q, root);
+        ntt_fwd_polys<LOGN, E, CAP, B>(sm, reinterpret_cast<u64(&)[1][E]>(r), tid, t, q, root);
         return;
     }
     constexpr int NFULL = LOGN / LE, TAIL = LOGN % LE;
@@ -546,7 +560,7 @@ __device__ __forceinline__ void ntt_fwd_regs(u64* sm, u64 (&r)[E], int tid, cons
         store_sm_rt<E>(sm, r, tid, LOGN - LE * NFULL);
         __syncthreads();
         load_sm<LOGN, LE * NFULL, E, false>(sm, r, tid);
-        fwd_regs<LOGN, LE * NFULL, E, false, CAP, CAP>(r, tid, t.tw, q, 1);
+        fwd_regs<LOGN, LE * NFULL, E, false, CAP, CAP>(reinterpret_cast<u64(&)[1][E]>(r), tid, t.tw, q, 1);
     }
 }
 

@@ -103,7 +103,9 @@ def test_products_and_bounds(tmp_path):
 @pytest.mark.gpu
 @pytest.mark.parametrize("ring", [
     dict(log_n=10, prime_bits=[60, 49, 50, 51], log2_scale=40, special_bits=61),
+    dict(log_n=11, prime_bits=[60, 50], log2_scale=40, special_bits=61),   # the polynomials in turn up to here
     dict(log_n=12, prime_bits=[51, 50], log2_scale=40, special_bits=61),
+    dict(log_n=13, prime_bits=[60, 49], log2_scale=40, special_bits=61),
     dict(log_n=14, prime_bits=[60, 50, 51], log2_scale=40, special_bits=61),
 ], ids=lambda r: "n%d" % (1 << r["log_n"]))
 def test_matching_against_the_oracle(ring):
