@@ -189,19 +189,10 @@ extern "C" ichee_status ichee_ctx_create(const ichee_params* p, int device, iche
     std::memset(&c->rns, 0, sizeof(c->rns));
     c->rns.logn = c->logn;
     c->rns.n_mod = c->nmod;
-    std::vector<u64> ninv(c->nmod);
+    std::vector<u64> ninv(c->nmod), tables(nwords);
     for (int m = 0; m < c->nmod; ++m) {
         const u64 qm = c->q[m];
-        const std::vector<u64> t = hm::twiddles(qm, (unsigned)c->logn);   // [tw | twp | itw | itwp]
-        std::vector<u64> pairs(t.size());                                     // [(tw, twp)] then [(itw, itwp)]
-        for (int d = 0; d < 2; ++d)
-            for (int k = 0; k < c->n; ++k) {
-                pairs[((size_t)d * c->n + k) * 2] = t[(size_t)(2 * d) * c->n + k];
-                pairs[((size_t)d * c->n + k) * 2 + 1] = t[(size_t)(2 * d + 1) * c->n + k];
-            }
-        if (cudaMemcpy(c->d_tables + (size_t)m * 4 * c->n, pairs.data(), pairs.size() * 8, cudaMemcpyHostToDevice) !=
-            cudaSuccess)
-            return cleanup(fail(ICHEE_ECUDA, "upload tables"));
+        hm::twiddle_pairs(qm, (unsigned)c->logn, tables.data() + (size_t)m * 4 * c->n);
         c->rns.q[m] = qm;
         c->rns.mu[m] = (u64)(((hm::u128)1 << 64) / qm);
         const hm::u128 big = ~(hm::u128)0 / qm;  // floor(2^128 / q): q is odd, so 2^128 - 1 gives the same
@@ -215,6 +206,8 @@ extern "C" ichee_status ichee_ctx_create(const ichee_params* p, int device, iche
         c->rns.tab[m].itw = reinterpret_cast<const ulonglong2*>(base + 2 * (size_t)c->n);
         ninv[m] = hm::invm((u64)c->n % qm, qm);
     }
+    if (cudaMemcpy(c->d_tables, tables.data(), nwords * 8, cudaMemcpyHostToDevice) != cudaSuccess)
+        return cleanup(fail(ICHEE_ECUDA, "upload tables"));
     if (cudaMalloc(&c->d_ninv, 8 * (size_t)c->nmod) != cudaSuccess) return cleanup(fail(ICHEE_ENOMEM, "ninv"));
     cudaMemcpy(c->d_ninv, ninv.data(), 8 * (size_t)c->nmod, cudaMemcpyHostToDevice);
 
@@ -343,23 +336,18 @@ static ichee_status make_aux(ichee_ctx* c)
     const size_t n = (size_t)c->n;
     if (cudaMalloc(&c->d_aux_tables, (size_t)c->aux.n * 2 * n * sizeof(uint2)) != cudaSuccess)
         return fail(ICHEE_ENOMEM, "auxiliary tables");
-    std::vector<uint2> t(2 * n);
+    std::vector<u64> pairs(4 * n);
+    std::vector<uint2> t((size_t)c->aux.n * 2 * n);
     for (int i = 0; i < c->aux.n; ++i) {
-        const u64 p = taken[i], psi = hm::root_2n(p, (unsigned)c->logn), psi_inv = hm::invm(psi, p);
-        u64 w = 1, iw = 1;
-        for (size_t k = 0; k < n; ++k) {
-            const unsigned r = hm::bitrev((unsigned)k, (unsigned)c->logn);
-            t[r] = make_uint2((u32)w, (u32)((w << 32) / p));
-            t[n + r] = make_uint2((u32)iw, (u32)((iw << 32) / p));
-            w = w * psi % p;
-            iw = iw * psi_inv % p;
-        }
-        uint2* d = c->d_aux_tables + (size_t)i * 2 * n;
-        if (cudaMemcpy(d, t.data(), 2 * n * sizeof(uint2), cudaMemcpyHostToDevice) != cudaSuccess)
-            return fail(ICHEE_ECUDA, "upload auxiliary tables");
+        hm::twiddle_pairs(taken[i], (unsigned)c->logn, pairs.data());
+        for (size_t k = 0; k < 2 * n; ++k)   // the 32-bit companion is the upper half of the 64-bit one
+            t[(size_t)i * 2 * n + k] = make_uint2((u32)pairs[2 * k], (u32)(pairs[2 * k + 1] >> 32));
+        const uint2* d = c->d_aux_tables + (size_t)i * 2 * n;
         c->aux.tw[i] = d;
         c->aux.itw[i] = d + n;
     }
+    if (cudaMemcpy(c->d_aux_tables, t.data(), t.size() * sizeof(uint2), cudaMemcpyHostToDevice) != cudaSuccess)
+        return fail(ICHEE_ECUDA, "upload auxiliary tables");
     return ICHEE_OK;
 }
 
