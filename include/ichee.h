@@ -583,7 +583,7 @@ ichee_status ichee_sqdiff_sum_noalloc(ichee_ctx* ctx, const uint64_t* d_a, const
  * Measurement utility (not part of the method): integer throughput of CUDA device `device`,
  * the context of the rooflines of the transform kernels. Runs two register-only kernels for a
  * few tens of milliseconds: 32-bit multiply-adds (*imad_per_s, operations per second over the
- * whole GPU) and the library's forward butterfly with its Shoup product on 60-bit residues
+ * whole GPU) and a textbook forward butterfly (exact Shoup quotient) on 60-bit residues
  * (*butterflies_per_s). Synchronous; allocates and frees a small output buffer. Errors: EINVAL,
  * ECUDA.
  */

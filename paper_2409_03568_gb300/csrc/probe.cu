@@ -1,6 +1,6 @@
 // probe.cu -- integer throughput of the GPU, measured: the context the rooflines of the
 // transform kernels need (their peak is derived from the SM count, clock and multiply-add rate;
-// this measures the rate and what the library's butterfly reaches on its own). Not part of
+// this measures the rate and what a textbook butterfly reaches on its own). Not part of
 // the method.
 #include "api_internal.h"
 #include "common.cuh"
@@ -26,8 +26,9 @@ __global__ void __launch_bounds__(512) k_probe_imad(u32* out, int iters)
     out[(size_t)blockIdx.x * blockDim.x + threadIdx.x] = acc;
 }
 
-// The library's forward butterfly (Harvey lazy reduction, Shoup product) on 16 residues held
-// in registers: four radix-2 stages per iteration, 32 butterflies.
+// A yardstick that stays the same while the kernels change: the 64-bit forward butterfly with an exact
+// Shoup quotient and one conditional subtraction (Harvey) on 16 residues held in registers, four radix-2
+// stages per iteration, 32 butterflies. The transforms' own butterflies are cheaper (ntt.cuh).
 __global__ void __launch_bounds__(512) k_probe_butterfly(u64* out, u64 q, u64 w, u64 wp, int iters)
 {
     u64 r[16];
