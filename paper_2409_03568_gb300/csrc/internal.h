@@ -15,6 +15,7 @@ constexpr int kAuxMax = 3;
 struct AuxPrimes {
     int n;                          // primes in use (2 or 3)
     u32 p[kAuxMax], pinv[kAuxMax];  // p^{-1} mod 2^32
+    u32 zero;                       // 0, as the third addend of a butterfly's sum (ntt32.cuh)
     const uint2* tw[kAuxMax];       // [N] psi^{bitrev(k)}
     const uint2* itw[kAuxMax];      // [N] psi^{-bitrev(k)}
 };

@@ -279,7 +279,7 @@ __global__ void __launch_bounds__(EncShape<LOGN>::T) k_pk_aux(const __grid_const
             const u32 m = (u32)((c > q / 2 ? q - c : c) % p);
             r[0][e] = c > q / 2 && m != 0 ? p - m : m;
         }
-        ntt32_fwd<LOGN, 1, E, false>(reinterpret_cast<u32*>(smem), r, tid, a.aux.tw[i], p);
+        ntt32_fwd<LOGN, 1, E, false>(reinterpret_cast<u32*>(smem), r, tid, a.aux.tw[i], p, a.aux.zero);
 #pragma unroll
         for (int e = 0; e < E; ++e)
             a.out[enc_pk_at<LOGN>(u, b, elem_index<LOGN, LAST, E>(tid, e))] = (u32)((u64)(r[0][e] % p) * k % p);
@@ -320,9 +320,9 @@ cudaError_t launch_pk_aux(const PkAuxArgs& a, int logn, int n_units, cudaStream_
 // k = round(sum_i y_i / p_i) is reduced modulo q_l by one 32-bit quotient estimate (enc_crt).
 // Three 64-bit transforms per limb become three 28-bit ones per ciphertext and four or six per limb
 // (19 at N = 2^13 with primes 60/40/60), at about a fifth of the multiply-pipe time each. Measured
-// against the 64-bit form: 4096 pixels at N = 2^13 3.03 -> 2.56 ms, 851 pixels at N = 2^14 and five
-// limbs 3.34 -> 1.77 ms, 1224 pixels at N = 2^12 0.66 -> 0.39 ms (there also more than one block per
-// SM). Bound by the integer multiply pipe (75 % busy), then by the exchanges between the passes.
+// against the 64-bit form: 4096 pixels at N = 2^13 3.03 -> 2.43 ms, 851 pixels at N = 2^14 and five
+// limbs 3.34 -> 1.69 ms, 1224 pixels at N = 2^12 0.66 -> 0.39 ms (there also more than one block per
+// SM). Bound by the integer multiply pipe (76 % busy), then by the exchanges between the passes.
 // ---------------------------------------------------------------------------------------
 
 // The sample word of a coefficient: v + 1 (bits 0-1), e0 + 32 (bits 2-7), e1 + 32 (bits 8-13).
@@ -414,7 +414,8 @@ __device__ __forceinline__ void encrypt_ct(const EncArgs& a, int group, int p, u
             u32 r[1][E];
 #pragma unroll
             for (int e = 0; e < E; ++e) r[0][e] = (u32)((int)(smp[x0 + elem_offset<LOGN, 0, E>(e)] & 3u) - 1);
-            ntt32_fwd<LOGN, 1, E, true>(ex + (S::BUFS == 2 ? turn * NP * N : 0), r, tid, a.aux.tw[i], a.aux.p[i]);
+            ntt32_fwd<LOGN, 1, E, true>(ex + (S::BUFS == 2 ? turn * NP * N : 0), r, tid, a.aux.tw[i], a.aux.p[i],
+                                        a.aux.zero);
             turn ^= 1;
 #pragma unroll
             for (int e = 0; e < E; ++e) vh[(i - i0) * N + e * T + tid] = r[0][e];
@@ -447,7 +448,8 @@ __device__ __forceinline__ void encrypt_ct(const EncArgs& a, int group, int p, u
                         }
                     }
                     if (S::BUFS == 1) __syncthreads();
-                    ntt32_inv<LOGN, NP, E>(ex + (S::BUFS == 2 ? turn * NP * N : 0), y, tid, a.aux.itw[i], pi);
+                    ntt32_inv<LOGN, NP, E>(ex + (S::BUFS == 2 ? turn * NP * N : 0), y, tid, a.aux.itw[i], pi,
+                                           a.aux.zero);
                     turn ^= 1;
                 }
                 u64* dst = ct + ((u64)pb * L + l) * N + x0;

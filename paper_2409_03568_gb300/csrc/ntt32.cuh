@@ -14,6 +14,12 @@
 // Ranges: p < 2^28, so sixteen multiples of p fit a word and most butterflies need no reduction.
 // The code knows every register's bound (a multiple of p) at compile time and folds a value below 2p
 // only when the next sum would pass 16 p.
+//
+// z is a zero that the compiler does not know. A sum of two words may be issued as a multiply-add on the
+// multiply pipe, which bounds these transforms; a sum of three takes the adder, half idle here. 4096
+// fresh encryptions at N = 2^13 2.50 -> 2.43 ms (the inverse alone 2.48), at 2^14 7.72 -> 7.53, at 2^12
+// 1.22 -> 1.21; the same in the reconstruction modulo q was slower (2.49), and the 64-bit transforms
+// gain nothing from it.
 #pragma once
 #include "internal.h"
 #include "ntt.cuh"
@@ -113,7 +119,7 @@ __host__ __device__ constexpr int fwd32_bound(int b, int S)
 // Forward stages S0 .. S0+S-1 on registers below B p. With TERNARY0 the registers of pass 0 hold
 // the integers -1, 0, 1 (as signed words).
 template <int LOGN, int S0, int NP, int E, int B, bool TERNARY0>
-__device__ __forceinline__ void fwd32_regs(u32 (&r)[NP][E], int tid, const uint2* __restrict__ tw, u32 p)
+__device__ __forceinline__ void fwd32_regs(u32 (&r)[NP][E], int tid, const uint2* __restrict__ tw, u32 p, u32 z)
 {
     using P = Pass<LOGN, S0, E>;
     const u32 p2 = p + p;
@@ -135,7 +141,7 @@ __device__ __forceinline__ void fwd32_regs(u32 (&r)[NP][E], int tid, const uint2
                     // ternary: the product is the signed integer 0 or +-w, and the sums with
                     // 2p lie in (0, 4p)
                     const u32 T = ternary ? r[n][i1] * w[b].x : shoup32(r[n][i1], w[b].x, w[b].y, p);
-                    r[n][i0] = ternary ? X + T + p2 : X + T;
+                    r[n][i0] = ternary ? X + T + p2 : X + T + z;
                     r[n][i1] = X - T + p2;
                 }
             });
@@ -144,15 +150,15 @@ __device__ __forceinline__ void fwd32_regs(u32 (&r)[NP][E], int tid, const uint2
 }
 
 template <int LOGN, int S0, int NP, int E, int B>
-__device__ __forceinline__ void fwd32_rest(u32* sm, u32 (&r)[NP][E], int tid, const uint2* __restrict__ tw, u32 p)
+__device__ __forceinline__ void fwd32_rest(u32* sm, u32 (&r)[NP][E], int tid, const uint2* __restrict__ tw, u32 p, u32 z)
 {
     constexpr int LE = Radix<E>::LE;
     if constexpr (S0 <= NttShape<LOGN, E>::LAST) {
         store_sm32<LOGN, S0 - LE, NP, E>(sm, r, tid);
         exchange_barrier<LOGN, S0, E>();
         load_sm32<LOGN, S0, NP, E>(sm, r, tid);
-        fwd32_regs<LOGN, S0, NP, E, B, false>(r, tid, tw, p);
-        fwd32_rest<LOGN, S0 + LE, NP, E, fwd32_bound(B, Pass<LOGN, S0, E>::S)>(sm, r, tid, tw, p);
+        fwd32_regs<LOGN, S0, NP, E, B, false>(r, tid, tw, p, z);
+        fwd32_rest<LOGN, S0 + LE, NP, E, fwd32_bound(B, Pass<LOGN, S0, E>::S)>(sm, r, tid, tw, p, z);
     }
 }
 
@@ -166,13 +172,13 @@ __host__ __device__ constexpr int fwd32_out()
 // Whole forward transform: input in the layout of pass 0 (ternary integers with TERNARY0, else
 // residues below p), output in the layout of the last pass, bit-reversed order, below 16 p.
 template <int LOGN, int NP, int E, bool TERNARY0>
-__device__ __forceinline__ void ntt32_fwd(u32* sm, u32 (&r)[NP][E], int tid, const uint2* __restrict__ tw, u32 p)
+__device__ __forceinline__ void ntt32_fwd(u32* sm, u32 (&r)[NP][E], int tid, const uint2* __restrict__ tw, u32 p, u32 z)
 {
     constexpr int LE = Radix<E>::LE;
     // bound entering pass 0: the ternary stage leaves 4, as a stage from 2 would
     constexpr int B0 = TERNARY0 ? 2 : 1;
-    fwd32_regs<LOGN, 0, NP, E, B0, TERNARY0>(r, tid, tw, p);
-    fwd32_rest<LOGN, LE, NP, E, fwd32_bound(B0, LE)>(sm, r, tid, tw, p);
+    fwd32_regs<LOGN, 0, NP, E, B0, TERNARY0>(r, tid, tw, p, z);
+    fwd32_rest<LOGN, LE, NP, E, fwd32_bound(B0, LE)>(sm, r, tid, tw, p, z);
 }
 
 // ---- inverse ------------------------------------------------------------------------------
@@ -196,7 +202,7 @@ __host__ __device__ constexpr int inv32_bound(int b, int S)
 
 // Inverse stages S0+S-1 .. S0 on registers below B p; the outputs of pass 0 are folded below 2p.
 template <int LOGN, int S0, int NP, int E, int B>
-__device__ __forceinline__ void inv32_regs(u32 (&r)[NP][E], int tid, const uint2* __restrict__ itw, u32 p)
+__device__ __forceinline__ void inv32_regs(u32 (&r)[NP][E], int tid, const uint2* __restrict__ itw, u32 p, u32 z)
 {
     using P = Pass<LOGN, S0, E>;
     const u32 p2 = p + p, neg_p2 = 0u - p2;
@@ -219,7 +225,7 @@ __device__ __forceinline__ void inv32_regs(u32 (&r)[NP][E], int tid, const uint2
                         X = fold32<bound>(X, p, neg_p2);
                         Y = fold32<bound>(Y, p, neg_p2);
                     }
-                    r[n][i0] = X + Y;
+                    r[n][i0] = X + Y + z;
                     r[n][i1] = shoup32(X - Y + add, w[b].x, w[b].y, p);
                 }
             });
@@ -234,24 +240,24 @@ __device__ __forceinline__ void inv32_regs(u32 (&r)[NP][E], int tid, const uint2
 }
 
 template <int LOGN, int S0, int NP, int E, int B>
-__device__ __forceinline__ void inv32_rest(u32* sm, u32 (&r)[NP][E], int tid, const uint2* __restrict__ itw, u32 p)
+__device__ __forceinline__ void inv32_rest(u32* sm, u32 (&r)[NP][E], int tid, const uint2* __restrict__ itw, u32 p, u32 z)
 {
     constexpr int LE = Radix<E>::LE;
-    inv32_regs<LOGN, S0, NP, E, B>(r, tid, itw, p);
+    inv32_regs<LOGN, S0, NP, E, B>(r, tid, itw, p, z);
     if constexpr (S0 > 0) {
         store_sm32<LOGN, S0, NP, E>(sm, r, tid);
         exchange_barrier<LOGN, S0, E>();
         load_sm32<LOGN, S0 - LE, NP, E>(sm, r, tid);
-        inv32_rest<LOGN, S0 - LE, NP, E, inv32_bound(B, Pass<LOGN, S0, E>::S)>(sm, r, tid, itw, p);
+        inv32_rest<LOGN, S0 - LE, NP, E, inv32_bound(B, Pass<LOGN, S0, E>::S)>(sm, r, tid, itw, p, z);
     }
 }
 
 // Whole inverse transform (without 1/N): input in the layout of the last pass, below 2p; output
 // in the layout of pass 0, natural order, below 2p.
 template <int LOGN, int NP, int E>
-__device__ __forceinline__ void ntt32_inv(u32* sm, u32 (&r)[NP][E], int tid, const uint2* __restrict__ itw, u32 p)
+__device__ __forceinline__ void ntt32_inv(u32* sm, u32 (&r)[NP][E], int tid, const uint2* __restrict__ itw, u32 p, u32 z)
 {
-    inv32_rest<LOGN, NttShape<LOGN, E>::LAST, NP, E, 2>(sm, r, tid, itw, p);
+    inv32_rest<LOGN, NttShape<LOGN, E>::LAST, NP, E, 2>(sm, r, tid, itw, p, z);
 }
 
 }  // namespace ichee
