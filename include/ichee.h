@@ -397,7 +397,8 @@ ichee_status ichee_tuned_shape(const ichee_ctx* ctx, uint32_t kind, uint32_t* th
  * Set the launch shape of a kernel kind (e.g. tuning results saved from an earlier run), or with
  * ICHEE_TUNE_SCHEDULE the encrypt + mean-filter schedule (threads = 1: fused kernel, 0: two
  * kernels; blocks_per_sm ignored). threads: 128, 256 or 512 (the fused kernel also 1024, decryption
- * 32 to 1024 in powers of two);
+ * 32 to 1024 in powers of two; 256 with blocks_per_sm 0, its default, lets the library choose by ring
+ * size and number of ciphertexts);
  * blocks_per_sm: 1..32 resident blocks per SM striding over the work, or 0 for one block per
  * work item. Results do not depend on shapes or schedule. Errors: EINVAL.
  */

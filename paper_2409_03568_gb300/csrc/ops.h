@@ -67,7 +67,7 @@ cudaError_t launch_rescale(const OpsArgs& a, cudaStream_t st);
 // staged: the bulk-copy form (input columns staged in shared memory), else the register walk
 cudaError_t launch_meanfilter3(const OpsArgs& a, bool staged, int num_sms, cudaStream_t st);
 cudaError_t launch_blend(const OpsArgs& a, cudaStream_t st);
-cudaError_t launch_decrypt(const DecArgs& a, int threads, cudaStream_t st);
+cudaError_t launch_decrypt(const DecArgs& a, const LaunchShape& ls, int num_sms, cudaStream_t st);
 
 // Ragged batches (SegTable items: ciphertexts, or mean-filter rows x chunks x polys x channels).
 // All segments share the level, the scale class and the constants of `a`.
