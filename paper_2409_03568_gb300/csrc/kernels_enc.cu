@@ -279,6 +279,7 @@ __global__ void __launch_bounds__(EncShape<LOGN>::T) k_pk_aux(const __grid_const
             const u32 m = (u32)((c > q / 2 ? q - c : c) % p);
             r[0][e] = c > q / 2 && m != 0 ? p - m : m;
         }
+        if (b > 0) __syncthreads();   // two forward transforms in a row: the first one's last loads are over
         ntt32_fwd<LOGN, 1, E, false>(reinterpret_cast<u32*>(smem), r, tid, a.aux.tw[i], p, a.aux.zero);
 #pragma unroll
         for (int e = 0; e < E; ++e)
