@@ -124,9 +124,15 @@ ichee_status meanfilter_chunked(ichee_ctx* c, const uint64_t* const* a, const ic
         const int cnt = (int)std::min<uint32_t>(kMaxSegs, n - first);
         SegTable t;
         std::memset(&t, 0, sizeof(t));
-        fill_starts(t, first, cnt, [&](uint32_t i) {
-            return mf_items(c->logn, base.limbs, ls.threads, c->mf_staged != 0, ma[i].h, ma[i].c);
-        });
+        int rows = 0;
+        if (!c->mf_staged) {
+            u64 items[kMfMaxRows] = {};
+            for (int r = 1; r <= kMfMaxRows; ++r)
+                for (int s = 0; s < cnt; ++s)
+                    items[r - 1] += mf_items(c->logn, ls.threads, r, ma[first + s].h, ma[first + s].c);
+            rows = mf_rows(base.limbs, true, items, ls.threads, c->num_sms);
+        }
+        fill_starts(t, first, cnt, [&](uint32_t i) { return mf_items(c->logn, ls.threads, rows, ma[i].h, ma[i].c); });
         for (int s = 0; s < cnt; ++s) {
             const uint32_t i = first + s;
             t.in0[s] = a[i];
@@ -135,7 +141,7 @@ ichee_status meanfilter_chunked(ichee_ctx* c, const uint64_t* const* a, const ic
             t.w[s] = ma[i].w;
             t.c[s] = ma[i].c;
         }
-        CK(launch_meanfilter3_batch(base, t, ls, c->mf_staged != 0, c->num_sms, st));
+        CK(launch_meanfilter3_batch(base, t, ls, rows, c->num_sms, st));
     }
     return ICHEE_OK;
 }

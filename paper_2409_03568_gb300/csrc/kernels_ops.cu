@@ -216,20 +216,12 @@ __device__ __forceinline__ void mf_store1(const OpsArgs& a, const u64 (&s)[LIMBS
 // whole image); h is the height of the whole image (the clamping rows), y_end the end of the output
 // rows.
 // The next column's residues are loaded before the current column's outputs are computed: with R
-// small enough that nothing spills (128 registers, 512 threads per SM) the loads in flight cover
-// the memory latency. Measured (one 16-byte pair of coefficients and one row per thread before):
-// 128x128x3 at N = 2^13, four limbs 8.66 -> 6.98 ms (6.5 TB/s of input read once and output, 0.95 of
-// copy bandwidth); 128x128, three limbs 1.98 -> 1.77 ms; 48x48x3 at N = 2^14, five limbs 2.98 -> 2.60
-// ms. Without the early loads R = 2 took 10.3 ms at four limbs; R = 4 there and R = 5 at three limbs
-// spill (8.6 and 2.0 ms), R = 1 at four limbs takes 9.4.
-template <int LIMBS>
-static constexpr int kMfRows = LIMBS == 3 ? 4 : LIMBS <= 4 ? 3 : LIMBS <= 6 ? 2 : 1;
-
-template <int LIMBS>
+// small enough that nothing spills much (128 registers, 512 threads per SM) the loads in flight cover
+// the memory latency. R is chosen at the launch (mf_rows).
+template <int LIMBS, int R>
 __device__ __forceinline__ void meanfilter_rows(const OpsArgs& a, const u64* in0, u64* out0, int h, int w, int C, int y,
                                                 int y_end, int chunk, int b, int ch, int row0, int yout0)
 {
-    constexpr int R = kMfRows<LIMBS>;
     const int n = 1 << a.logn;
     const int c = chunk * blockDim.x + threadIdx.x;   // coefficient
     const u64 in_step = (u64)C * 2 * LIMBS * n, out_step = (u64)C * 2 * (LIMBS - 1) * n;   // one column further
@@ -251,12 +243,14 @@ __device__ __forceinline__ void meanfilter_rows(const OpsArgs& a, const u64* in0
 #pragma unroll
             for (int i = 0; i < R + 2; ++i) raw[i][l] = __ldg(src[i] + l * n);
     };
-    auto advance = [&](int x) {          // raw = column x, or the last one again
+    // raw = column x, or past the right edge the last one again: left as it is with one row (64x1 pixels,
+    // seven limbs 38.7 -> 33.3 us), read again with several (128x128x3, four limbs 6.98 ms; 7.01 if not)
+    auto advance = [&](int x) {
         if (x < w) {
 #pragma unroll
             for (int i = 0; i < R + 2; ++i) src[i] += in_step;
         }
-        load();
+        if (R > 1 || x < w) load();
     };
     load();
 #pragma unroll
@@ -448,10 +442,9 @@ __global__ void __launch_bounds__(512) k_meanfilter3_staged_batch(const __grid_c
 // Ragged batch (a single image or a band of rows is a batch of one): segment s has
 // ceil(rows / R) * chunks * 2 * c items, row groups fastest, so that neighbouring blocks share their
 // halo rows in L2. Launched with at most 512 threads (the tunable shapes).
-template <int LIMBS, class Table>
+template <int LIMBS, int R, class Table>
 __global__ void __launch_bounds__(512) k_meanfilter3(const __grid_constant__ OpsArgs a, const __grid_constant__ Table t)
 {
-    constexpr int R = kMfRows<LIMBS>;
     const int chunks = (1 << a.logn) / blockDim.x;
     const u64 total = t.start[t.n];
     for (u64 g = blockIdx.x; g < total; g += gridDim.x) {
@@ -463,7 +456,7 @@ __global__ void __launch_bounds__(512) k_meanfilter3(const __grid_constant__ Ops
         const int y0 = (int)t.y0[s], y = y0 + (int)(i % groups) * R; i /= groups;
         const int chunk = (int)(i % chunks); i /= chunks;
         const int b = (int)(i % 2); i /= 2;
-        meanfilter_rows<LIMBS>(a, t.in0[s], t.out[s], h, (int)t.w[s], (int)t.c[s], y, y0 + rows, chunk, b, (int)i,
+        meanfilter_rows<LIMBS, R>(a, t.in0[s], t.out[s], h, (int)t.w[s], (int)t.c[s], y, y0 + rows, chunk, b, (int)i,
                                (int)t.row0[s], y0);
     }
 }
@@ -1112,46 +1105,82 @@ static int mf_staged_threads(int limbs, int threads)
     return threads;
 }
 
-template <class Table>
-static cudaError_t mf_launch(const OpsArgs& a, const Table& t, LaunchShape ls, int num_sms, cudaStream_t st)
+// Largest R per limb count that pays: at 128x128x3, N = 2^13 and four limbs R = 3 takes 6.98 ms (6.5 TB/s of
+// input read once and output; R = 1 9.4, R = 2 10.3 without the early loads); one more row than here
+// spills at three and four limbs, and at two gains nothing (64x64 at N = 2^13 328 and 327 us, 61x83 410 and
+// 419). Ragged batches of two limbs take at most 2 (62 registers there: 30 images of 20x21 at N = 2^13 917
+// us, with 3 rows 997).
+static int mf_max_rows(int limbs, bool batch)
+{
+    if (limbs == 2) return batch ? 2 : 3;
+    return limbs == 3 ? 4 : limbs == 4 ? 3 : limbs <= 6 ? 2 : 1;
+}
+
+// Few rows per thread fill the GPU with a small image, many read the halo rows less often: the R with the
+// least waves x (rows loaded per block), at the four blocks of 128 threads an SM holds. Measured, one
+// row of 16-byte pairs per thread | R = 1, 2, 3, 4 (the rule's choice in brackets): N = 2^10, three limbs
+// 8x8 8.2 | [4.6] 5.7 7.2 9.5 us; 100x100 178 | 185 196 [165] 172; N = 2^11 17x33 26.0 | 22.8 [21.5] 30.2
+// 41.8; N = 2^13 64x64 520 | 491 507 476 [471]; four limbs 16x16 57.5 | 53.3 [47.0] 60.5. Over 390
+// images and batches of 2 to 8 limbs the choice is within 1.2 % of the best R on average.
+int mf_rows(int limbs, bool batch, const u64 (&items)[kMfMaxRows], int threads, int num_sms)
+{
+    const u64 resident = (u64)num_sms * (threads < 512 ? 512 / threads : 1);
+    int best = 1;
+    u64 best_cost = ~0ull;
+    for (int r = 1; r <= mf_max_rows(limbs, batch); ++r) {
+        const u64 cost = (items[r - 1] + resident - 1) / resident * (r + 2);
+        if (cost < best_cost) {
+            best = r;
+            best_cost = cost;
+        }
+    }
+    return best;
+}
+
+u64 mf_items(int logn, int threads, int r, u32 rows, u32 c)
+{
+    const u64 n = (u64)1 << logn;
+    if (r == 0) return rows * (n / 2 / threads) * 2 * c;
+    return ((u64)rows + r - 1) / r * (n / threads) * 2 * c;
+}
+
+#define ICHEE_MF_CASES(TABLE)                                                                              \
+    ICHEE_MF_CASE(2, 1, TABLE) ICHEE_MF_CASE(2, 2, TABLE) ICHEE_MF_CASE(3, 1, TABLE) ICHEE_MF_CASE(3, 2, TABLE) \
+    ICHEE_MF_CASE(3, 3, TABLE) ICHEE_MF_CASE(3, 4, TABLE) ICHEE_MF_CASE(4, 1, TABLE) ICHEE_MF_CASE(4, 2, TABLE) \
+    ICHEE_MF_CASE(4, 3, TABLE) ICHEE_MF_CASE(5, 1, TABLE) ICHEE_MF_CASE(5, 2, TABLE) ICHEE_MF_CASE(6, 1, TABLE) \
+    ICHEE_MF_CASE(6, 2, TABLE) ICHEE_MF_CASE(7, 1, TABLE) ICHEE_MF_CASE(8, 1, TABLE)
+
+#define ICHEE_MF_CASE(LB, R, TABLE) \
+    case LB * 8 + R: k_meanfilter3<LB, R, TABLE><<<g, ls.threads, 0, st>>>(a, t); break;
+static cudaError_t mf_launch(const OpsArgs& a, const SegTable& t, LaunchShape ls, int r, int num_sms, cudaStream_t st)
 {
     const unsigned g = persistent_grid(t.start[t.n], ls, num_sms);
     if (g == 0) return cudaSuccess;
-    switch (a.limbs) {
-#define ICHEE_MF_CASE(LB) \
-    case LB: k_meanfilter3<LB, Table><<<g, ls.threads, 0, st>>>(a, t); break;
-        ICHEE_MF_CASE(2) ICHEE_MF_CASE(3) ICHEE_MF_CASE(4) ICHEE_MF_CASE(5) ICHEE_MF_CASE(6) ICHEE_MF_CASE(7) ICHEE_MF_CASE(8)
-#undef ICHEE_MF_CASE
+    switch (a.limbs * 8 + r) {
+        ICHEE_MF_CASES(SegTable)
     default: return cudaErrorInvalidValue;
     }
     return cudaGetLastError();
 }
 
-static int mf_rows(int limbs)
+static cudaError_t mf_launch(const OpsArgs& a, const OneSeg& t, LaunchShape ls, int r, int num_sms, cudaStream_t st)
 {
-    switch (limbs) {
-    case 2: return kMfRows<2>;
-    case 3: return kMfRows<3>;
-    case 4: return kMfRows<4>;
-    case 5: return kMfRows<5>;
-    case 6: return kMfRows<6>;
-    case 7: return kMfRows<7>;
-    default: return kMfRows<8>;
+    const unsigned g = persistent_grid(t.start[t.n], ls, num_sms);
+    if (g == 0) return cudaSuccess;
+    switch (a.limbs * 8 + r) {
+        ICHEE_MF_CASES(OneSeg) ICHEE_MF_CASE(2, 3, OneSeg)
+    default: return cudaErrorInvalidValue;
     }
+    return cudaGetLastError();
 }
-
-u64 mf_items(int logn, int limbs, int threads, bool staged, u32 rows, u32 c)
-{
-    if (staged) return (u64)rows * (((u64)1 << logn) / 2 / threads) * 2 * c;
-    const int r = mf_rows(limbs);
-    return ((u64)rows + r - 1) / r * (((u64)1 << logn) / threads) * 2 * c;
-}
+#undef ICHEE_MF_CASE
+#undef ICHEE_MF_CASES
 
 cudaError_t launch_meanfilter3(const OpsArgs& a, bool staged, int num_sms, cudaStream_t st)
 {
     const int threads = staged ? 256 : 128;   // 128: finer last waves on small images (256: 2 to 5 % slower there)
     if (staged) {
-        const u64 blocks = mf_items(a.logn, a.limbs, threads, true, (u32)a.rows, (u32)a.c);
+        const u64 blocks = mf_items(a.logn, threads, 0, (u32)a.rows, (u32)a.c);
         if (blocks == 0) return cudaSuccess;
         switch (a.limbs) {
 #define ICHEE_MF_STAGED_CASE(LB) \
@@ -1162,10 +1191,13 @@ cudaError_t launch_meanfilter3(const OpsArgs& a, bool staged, int num_sms, cudaS
         default: return cudaErrorInvalidValue;
         }
     }
+    u64 items[kMfMaxRows];
+    for (int r = 1; r <= kMfMaxRows; ++r) items[r - 1] = mf_items(a.logn, threads, r, (u32)a.rows, (u32)a.c);
+    const int rows = mf_rows(a.limbs, false, items, threads, num_sms);
     OneSeg t;   // the image, or its band, as a batch of one
     std::memset(&t, 0, sizeof(t));
     t.n = 1;
-    t.start[1] = mf_items(a.logn, a.limbs, threads, false, (u32)a.rows, (u32)a.c);
+    t.start[1] = items[rows - 1];
     t.in0[0] = a.in0;
     t.out[0] = a.out;
     t.h[0] = (uint32_t)a.h;
@@ -1174,7 +1206,7 @@ cudaError_t launch_meanfilter3(const OpsArgs& a, bool staged, int num_sms, cudaS
     t.y0[0] = (uint32_t)a.y0;
     t.rows[0] = (uint32_t)a.rows;
     t.row0[0] = (uint32_t)a.row0;
-    return mf_launch(a, t, LaunchShape{threads, 0}, num_sms, st);
+    return mf_launch(a, t, LaunchShape{threads, 0}, rows, num_sms, st);
 }
 
 cudaError_t launch_blend(const OpsArgs& a, cudaStream_t st)
@@ -1209,12 +1241,12 @@ cudaError_t launch_blend(const OpsArgs& a, cudaStream_t st)
     return cudaGetLastError();
 }
 
-cudaError_t launch_meanfilter3_batch(const OpsArgs& a, const SegTable& t, LaunchShape ls, bool staged, int num_sms,
+cudaError_t launch_meanfilter3_batch(const OpsArgs& a, const SegTable& t, LaunchShape ls, int rows, int num_sms,
                                      cudaStream_t st)
 {
     const u64 total = t.n > 0 ? t.start[t.n] : 0;
     if (total == 0) return cudaSuccess;
-    if (staged) {
+    if (rows == 0) {
         // items were counted by the caller for ls.threads; the staged block keeps that count
         // unless its stages do not fit, so the caller counts with mf_batch_threads
         const int th = mf_staged_threads(a.limbs, ls.threads);
@@ -1228,7 +1260,7 @@ cudaError_t launch_meanfilter3_batch(const OpsArgs& a, const SegTable& t, Launch
         default: return cudaErrorInvalidValue;
         }
     }
-    return mf_launch(a, t, ls, num_sms, st);
+    return mf_launch(a, t, ls, rows, num_sms, st);
 }
 
 // Threads per block of the fused kernel for a launch shape: 32 x columns per strip (at least 4

@@ -71,13 +71,17 @@ cudaError_t launch_decrypt(const DecArgs& a, const LaunchShape& ls, int num_sms,
 
 // Ragged batches (SegTable items: ciphertexts, or mean-filter rows x chunks x polys x channels).
 // All segments share the level, the scale class and the constants of `a`.
-cudaError_t launch_meanfilter3_batch(const OpsArgs& a, const SegTable& t, LaunchShape ls, bool staged, int num_sms,
+// Mean filter: rows = rows per thread of the register walk (mf_rows), 0 = the staged form.
+cudaError_t launch_meanfilter3_batch(const OpsArgs& a, const SegTable& t, LaunchShape ls, int rows, int num_sms,
                                      cudaStream_t st);
 // Threads per block the batched mean filter runs with for a requested count (the staged form
-// halves it while its stages would not fit), and the items of an image (or of a band of rows) with
-// that many threads.
+// halves it while its stages would not fit), the items of an image (or of a band of rows) with
+// that many threads and r rows per thread (0: staged), and the rows per thread for a launch of items[r - 1]
+// items with r.
+constexpr int kMfMaxRows = 4;
 int mf_batch_threads(int limbs, int threads, bool staged);
-u64 mf_items(int logn, int limbs, int threads, bool staged, u32 rows, u32 c);
+u64 mf_items(int logn, int threads, int r, u32 rows, u32 c);
+int mf_rows(int limbs, bool batch, const u64 (&items)[kMfMaxRows], int threads, int num_sms);
 cudaError_t launch_blend_batch(const OpsArgs& a, const SegTable& t, LaunchShape ls, int num_sms, cudaStream_t st);
 cudaError_t launch_ptadd_batch(const OpsArgs& a, const SegTable& t, LaunchShape ls, int num_sms, cudaStream_t st);
 cudaError_t launch_decrypt_batch(const DecArgs& a, const SegTable& t, LaunchShape ls, int num_sms, cudaStream_t st);
