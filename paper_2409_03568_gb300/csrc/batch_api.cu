@@ -429,9 +429,10 @@ extern "C" ichee_status ichee_autotune_batch(ichee_ctx* c, const ichee_cache* k,
         metas[i].level = (u32)(c->L - 1);
         metas[i].scale = c->delta;
     }
-    // blocks_per_sm = 0: one block per work item, the launch shape of the single-image kernels
+    // blocks_per_sm = 0: one block per work item, the launch shape of the single-image kernels. Every
+    // default is among the candidates, so that tuning cannot leave a context slower than it was.
     const LaunchShape cands[] = {{128, 4}, {128, 8}, {128, 16}, {256, 2}, {256, 4}, {256, 8},
-                                 {512, 1}, {512, 2}, {512, 4}, {256, 0}, {512, 0}};
+                                 {512, 1}, {512, 2}, {512, 4}, {128, 0}, {256, 0}, {512, 0}};
     uint32_t nrep = 0;
     const uint32_t cap = n_report ? *n_report : 0;
     auto time_it = [&](auto&& run, float* best) -> ichee_status {

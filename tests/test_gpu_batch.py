@@ -242,6 +242,23 @@ def test_fused_encrypt_meanfilter_equals_two_steps(ichee, ctx8192, base, randomi
         ichee.ichee_set_tuned_shape(ctx.handle, ichee.TUNE_SCHEDULE, saved)
 
 
+@pytest.mark.parametrize("kind", ["CACHE_RADIX", "CACHE_FULL"])
+def test_autotuner_times_the_defaults(ichee, kind):
+    """An untuned context's shapes are among the candidates, so that tuning can keep them."""
+    ctx = ichee.Context(10, [30, 30], 25)
+    ctx.keygen(3)
+    cache = ctx.build_cache(getattr(ichee, kind), 5, **({"radix_base": 16} if kind == "CACHE_RADIX" else {}))
+    kinds = [ichee.TUNE_MEANFILTER] + ([ichee.TUNE_RADIX, ichee.TUNE_FUSED] if kind == "CACHE_RADIX" else [ichee.TUNE_LOOKUP])
+    defaults = [(k,) + tuple(ichee.ichee_tuned_shape(ctx.handle, k)) for k in kinds]
+    px = torch.zeros(6, dtype=torch.uint8, device="cuda")
+    rep = ichee.ichee_autotune_batch(ctx.handle, cache, [px], [(2, 3, 1)], [1], [ctx.empty_cts(6, 1)], [ctx.empty_cts(6, 0)],
+                                     ctx.stream())
+    timed = {tuple(e[:3]) for e in rep}
+    assert timed.issuperset(defaults)
+    assert all((k,) + tuple(ichee.ichee_tuned_shape(ctx.handle, k)) in timed for k in kinds)
+    ctx.close()
+
+
 def test_set_tuned_shape_checks(ichee, ctx8192):
     ctx = ctx8192
     for args in ((ichee.TUNE_RADIX, 1024, 2), (ichee.TUNE_FUSED, 2048, 1), (ichee.TUNE_RADIX, 256, 33),
