@@ -397,10 +397,12 @@ ichee_status ichee_tuned_shape(const ichee_ctx* ctx, uint32_t kind, uint32_t* th
  * Set the launch shape of a kernel kind (e.g. tuning results saved from an earlier run), or with
  * ICHEE_TUNE_SCHEDULE the encrypt + mean-filter schedule (threads = 1: fused kernel, 0: two
  * kernels; blocks_per_sm ignored). threads: 128, 256 or 512 (the fused kernel also 1024, decryption
- * 32 to 1024 in powers of two; 256 with blocks_per_sm 0, its default, lets the library choose by ring
- * size and number of ciphertexts);
+ * 32 to 1024 in powers of two);
  * blocks_per_sm: 1..32 resident blocks per SM striding over the work, or 0 for one block per
  * work item. Results do not depend on shapes or schedule. Errors: EINVAL.
+ * Decryption: until a shape is set (ichee_tuned_shape gives 256 and 0) the library chooses the threads
+ * by ring size and number of ciphertexts. Of a set shape the single-image calls take the threads
+ * only, and 1024 below 64 ciphertexts.
  */
 ichee_status ichee_set_tuned_shape(ichee_ctx* ctx, uint32_t kind, uint32_t threads, uint32_t blocks_per_sm);
 

@@ -121,7 +121,8 @@ struct ichee_ctx {
     // one block per work item by default (the autotuner's choice for the 32-image batch)
     LaunchShape shape_radix = {256, 0}, shape_lookup = {256, 0}, shape_meanfilter = {128, 0};
     int mf_staged = 0;   // mean filter: 0 = register walk, 1 = bulk-copy staged form (ICHEE_TUNE_MF_STAGED)
-    LaunchShape shape_blend = {256, 0}, shape_ptadd = {256, 0}, shape_decrypt = {256, 0};
+    LaunchShape shape_blend = {256, 0}, shape_ptadd = {256, 0};
+    LaunchShape shape_decrypt = {0, 0};   // 0 threads: none set, the launch chooses
     LaunchShape shape_fused = {1024, 1};
     int fused_schedule = 0;   // ichee_encrypt_meanfilter_batch: 0 = two batched kernels, 1 = fused kernel
 };

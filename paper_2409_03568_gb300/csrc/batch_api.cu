@@ -529,7 +529,7 @@ extern "C" ichee_status ichee_tuned_shape(const ichee_ctx* c, uint32_t kind, uin
     case ICHEE_TUNE_LOOKUP: ls = c->shape_lookup; break;
     case ICHEE_TUNE_MEANFILTER: ls = c->shape_meanfilter; break;
     case ICHEE_TUNE_FUSED: ls = c->shape_fused; break;
-    case ICHEE_TUNE_DECRYPT: ls = c->shape_decrypt; break;
+    case ICHEE_TUNE_DECRYPT: ls = c->shape_decrypt.threads ? c->shape_decrypt : LaunchShape{256, 0}; break;
     case ICHEE_TUNE_SCHEDULE: *threads = (uint32_t)c->fused_schedule; *blocks_per_sm = 0; return ICHEE_OK;
     case ICHEE_TUNE_MF_STAGED: *threads = (uint32_t)c->mf_staged; *blocks_per_sm = 0; return ICHEE_OK;
     default: return fail(ICHEE_EINVAL, "unknown kernel kind %u", kind);

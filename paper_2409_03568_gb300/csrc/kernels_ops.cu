@@ -1329,35 +1329,20 @@ cudaError_t launch_ptadd_batch(const OpsArgs& a, const SegTable& t, LaunchShape 
     return cudaGetLastError();
 }
 
-// Threads of a block, one ciphertext each, when the caller set no shape of its own: with few ciphertexts
-// to an SM as many as keep its loads in flight, with many small ones as few as finish their rounds of four
-// loads together. Whole calls: N = 2^13, three limbs, one ciphertext per SM 19.3 us with 256 threads, 12.7
-// with 512 (two per SM 23.0 and 18.7, three 24.9 and 25.0); N = 2^14, five limbs, one per SM 58.0, 1024
-// threads 25.7; four per SM 76.5, 512 threads 73.6, seven 113.7 and 121.5; N = 2^12 2000 ciphertexts 43.4,
-// 128 threads 41.0 (608: 18.8 and 20.8); N = 2^10 4096 ciphertexts 34.0, 128 threads 21.1.
-static int decrypt_threads(int logn, u64 n_ct, const LaunchShape& ls, int num_sms)
-{
-    if (ls.threads != 256 || ls.blocks_per_sm != 0) return ls.threads;
-    const u64 per_sm = (n_ct + num_sms - 1) / num_sms, n = u64(1) << logn;
-    if (per_sm <= 1) return n / 8 < 1024 ? (int)(n / 8) : 1024;
-    if (logn >= 13) return per_sm <= n >> 12 ? 512 : 256;
-    return per_sm > 3 * (n >> 11) ? 128 : 256;
-}
-
 cudaError_t launch_decrypt_batch(const DecArgs& a, const SegTable& t, LaunchShape ls, int num_sms, cudaStream_t st)
 {
     const u64 total = t.n > 0 ? t.start[t.n] : 0;
     if (total == 0) return cudaSuccess;
-    ls.threads = decrypt_threads(a.logn, total, ls, num_sms);
+    ls.threads = decrypt_threads(a.logn, total, ls.threads, true, num_sms);
     if (ls.threads <= 256) k_decrypt_batch<256, 8><<<persistent_grid(total, ls, num_sms), ls.threads, 0, st>>>(a, t);
     else k_decrypt_batch<1024, 1><<<persistent_grid(total, ls, num_sms), ls.threads, 0, st>>>(a, t);
     return cudaGetLastError();
 }
 
-cudaError_t launch_decrypt(const DecArgs& a, const LaunchShape& ls, int num_sms, cudaStream_t st)
+cudaError_t launch_decrypt(const DecArgs& a, int threads, int num_sms, cudaStream_t st)
 {
     if (a.n_ct == 0) return cudaSuccess;
-    const int threads = decrypt_threads(a.logn, a.n_ct, {ls.threads, 0}, num_sms);
+    threads = decrypt_threads(a.logn, a.n_ct, threads, false, num_sms);
     if (threads < 32 || threads > 1024 || threads % 32 != 0) return cudaErrorInvalidValue;
     unsigned grid = (unsigned)(a.n_ct < (1u << 30) ? a.n_ct : (1u << 30));
     if (threads <= 256) k_decrypt<256, 8><<<grid, threads, 0, st>>>(a);

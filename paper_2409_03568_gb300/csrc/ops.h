@@ -60,6 +60,23 @@ struct DecArgs {
     u64* residues_out;             // optional [n_ct][nl]
 };
 
+// Threads of a block, one ciphertext each, when the caller set no shape of its own: with few ciphertexts
+// to an SM as many as keep its loads in flight, with many small ones as few as finish their rounds of four
+// loads together. Whole calls: N = 2^13, three limbs, one ciphertext per SM 19.3 us with 256 threads, 12.7
+// with 512 (two per SM 23.0 and 18.7, three 24.9 and 25.0); N = 2^14, five limbs, one per SM 58.0, 1024
+// threads 25.7; four per SM 76.5, 512 threads 73.6, seven 113.7 and 121.5; N = 2^12 2000 ciphertexts 43.4,
+// 128 threads 41.0 (608: 18.8 and 20.8); N = 2^10 4096 ciphertexts 34.0, 128 threads 21.1.
+// A shape that the caller set is taken as it is, but in a single-image call below 64 ciphertexts, where
+// one wide block each is meant.
+inline int decrypt_threads(int logn, u64 n_ct, int set, bool batch, int num_sms)
+{
+    if (set != 0) return !batch && n_ct < 64 ? 1024 : set;
+    const u64 per_sm = (n_ct + num_sms - 1) / num_sms, n = u64(1) << logn;
+    if (per_sm <= 1) return n / 8 < 1024 ? (int)(n / 8) : 1024;
+    if (logn >= 13) return per_sm <= n >> 12 ? 512 : 256;
+    return per_sm > 3 * (n >> 11) ? 128 : 256;
+}
+
 cudaError_t launch_addsub(const OpsArgs& a, bool subtract, cudaStream_t st);
 cudaError_t launch_ptadd(const OpsArgs& a, cudaStream_t st);
 cudaError_t launch_ptmul(const OpsArgs& a, cudaStream_t st);
@@ -67,7 +84,8 @@ cudaError_t launch_rescale(const OpsArgs& a, cudaStream_t st);
 // staged: the bulk-copy form (input columns staged in shared memory), else the register walk
 cudaError_t launch_meanfilter3(const OpsArgs& a, bool staged, int num_sms, cudaStream_t st);
 cudaError_t launch_blend(const OpsArgs& a, cudaStream_t st);
-cudaError_t launch_decrypt(const DecArgs& a, const LaunchShape& ls, int num_sms, cudaStream_t st);
+// threads (in the batch: ls.threads) as the caller set them, 0 if not.
+cudaError_t launch_decrypt(const DecArgs& a, int threads, int num_sms, cudaStream_t st);
 
 // Ragged batches (SegTable items: ciphertexts, or mean-filter rows x chunks x polys x channels).
 // All segments share the level, the scale class and the constants of `a`.
