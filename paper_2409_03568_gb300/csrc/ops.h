@@ -62,17 +62,19 @@ struct DecArgs {
 
 // Threads of a block, one ciphertext each, when the caller set no shape of its own: with few ciphertexts
 // to an SM as many as keep its loads in flight, with many small ones as few as finish their rounds of four
-// loads together. Whole calls: N = 2^13, three limbs, one ciphertext per SM 19.3 us with 256 threads, 12.7
-// with 512 (two per SM 23.0 and 18.7, three 24.9 and 25.0); N = 2^14, five limbs, one per SM 58.0, 1024
-// threads 25.7; four per SM 76.5, 512 threads 73.6, seven 113.7 and 121.5; N = 2^12 2000 ciphertexts 43.4,
-// 128 threads 41.0 (608: 18.8 and 20.8); N = 2^10 4096 ciphertexts 34.0, 128 threads 21.1.
+// loads together. GPU time of a call in us by threads: at most one ciphertext per SM, N = 2^10 and two limbs
+// 128: 5.0, 256: 5.1, 512: 5.9; N = 2^12, three limbs 256: 12.3, 512: 8.7, 1024: 11.4; N = 2^13, three limbs
+// 256: 20.2, 512: 11.6, 1024: 11.9; N = 2^14, five limbs 256: 57.0, 512: 26.3, 1024: 23.4. Two per SM at
+// 2^13 256: 21.9, 512: 16.6, three 22.3 and 22.2, four 26.5 and 29.1; four per SM at 2^14 256: 75.6, 512:
+// 72.0; whole calls of seven there 113.7 and 121.5. Many small ones, whole calls: N = 2^12, 2000
+// ciphertexts 256: 43.4, 128: 41.0 (608: 18.8 and 20.8); N = 2^10, 4096 ciphertexts 34.0 and 21.1.
 // A shape that the caller set is taken as it is, but in a single-image call below 64 ciphertexts, where
 // one wide block each is meant.
 inline int decrypt_threads(int logn, u64 n_ct, int set, bool batch, int num_sms)
 {
     if (set != 0) return !batch && n_ct < 64 ? 1024 : set;
     const u64 per_sm = (n_ct + num_sms - 1) / num_sms, n = u64(1) << logn;
-    if (per_sm <= 1) return n / 8 < 1024 ? (int)(n / 8) : 1024;
+    if (per_sm <= 1) return logn >= 13 ? (int)(n / 16) : (int)(n / 8);
     if (logn >= 13) return per_sm <= n >> 12 ? 512 : 256;
     return per_sm > 3 * (n >> 11) ? 128 : 256;
 }
