@@ -1160,7 +1160,7 @@ extern "C" ichee_status ichee_eval(ichee_ctx* c, ichee_op op, const uint64_t* d_
         set_rescale(c, a);
         fold_constants(c, a);
         a.c_w = (int)mb->c;
-        CK(launch_blend(a, st));
+        CK(launch_blend(a, c->num_sms, st));
         m.level = ma->level - 1;
         m.scale = ma->scale * c->delta / (double)c->q[ma->level];
         break;

@@ -1209,14 +1209,11 @@ cudaError_t launch_meanfilter3(const OpsArgs& a, bool staged, int num_sms, cudaS
     return mf_launch(a, t, LaunchShape{threads, 0}, rows, num_sms, st);
 }
 
-cudaError_t launch_blend(const OpsArgs& a, cudaStream_t st)
+cudaError_t launch_blend(const OpsArgs& a, int num_sms, cudaStream_t st)
 {
     if (a.limbs >= 4 && a.c_w == 1 && a.c > 1) {   // both forms measured at k_blend_shared
-        // coefficients shared out until the grid has a few blocks per SM
-        const u64 px2 = a.n_ct / a.c * 2;
-        int splits = 1;
-        while (px2 * splits < 152 * 16 && ((1 << a.logn) / splits) > 256) splits *= 2;
-        const u64 units = px2 * splits;
+        const int splits = blend_splits(a.logn, a.n_ct / a.c, num_sms);
+        const u64 units = a.n_ct / a.c * 2 * splits;
         const unsigned g = (unsigned)(units < (1u << 30) ? units : (1u << 30));
         switch (a.limbs) {
 #define ICHEE_BLEND_CASE(LB) \

@@ -85,7 +85,16 @@ cudaError_t launch_ptmul(const OpsArgs& a, cudaStream_t st);
 cudaError_t launch_rescale(const OpsArgs& a, cudaStream_t st);
 // staged: the bulk-copy form (input columns staged in shared memory), else the register walk
 cudaError_t launch_meanfilter3(const OpsArgs& a, bool staged, int num_sms, cudaStream_t st);
-cudaError_t launch_blend(const OpsArgs& a, cudaStream_t st);
+// Shares of a polynomial's coefficients in the blend with a one-channel pattern: twice as many until the
+// grid has 16 blocks per SM or a share is one coefficient per thread (N = 2^13, four limbs, against the form
+// with a block per ciphertext and polynomial: 1x1x3 19.9 -> 3.9 us, 4x4x3 23.6 -> 12.2, 16x16x3 170 -> 150).
+inline int blend_splits(int logn, u64 pixels, int num_sms)
+{
+    int splits = 1;
+    while (pixels * 2 * splits < (u64)num_sms * 16 && ((1 << logn) / splits) > 256) splits *= 2;
+    return splits;
+}
+cudaError_t launch_blend(const OpsArgs& a, int num_sms, cudaStream_t st);
 // threads (in the batch: ls.threads) as the caller set them, 0 if not.
 cudaError_t launch_decrypt(const DecArgs& a, int threads, int num_sms, cudaStream_t st);
 

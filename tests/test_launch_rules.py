@@ -31,13 +31,22 @@ int main()
     for (int logn = 10; logn <= 14; ++logn)
         for (u64 n : {1ull, 152ull})
             if (decrypt_threads(logn, n, 0, false, 152) != fastest[logn - 10]) ++bad;
+    // blend with a one-channel pattern: 16 blocks per SM, whatever their number, or 256 coefficients a share
+    for (int sms : {76, 152, 304})
+        for (int logn = 10; logn <= 14; ++logn)
+            for (u64 px : {1ull, 30ull, 300ull, 3000ull}) {
+                const u64 s = blend_splits(logn, px, sms), n = 1ull << logn;
+                if (2 * px * s < 16ull * sms && n / s > 256) ++bad;
+                if (s > 1 && px * s >= 16ull * sms) ++bad;   // half as many would do
+                if (n % s || n / s < 256) ++bad;
+            }
     std::printf("bad %d\n", bad);
     return bad != 0;
 }
 """
 
 
-def test_decryption_threads(tmp_path):
+def test_launch_rules(tmp_path):
     cc = nvcc()
     if cc is None:
         pytest.skip("nvcc not found")
