@@ -115,6 +115,9 @@ inline uint32_t __viaddmin_u32(uint32_t a, uint32_t b, uint32_t c) { const uint3
 template <class T> inline T __ldg(const T* p) { return *p; }
 template <class T> inline T __ldcs(const T* p) { return *p; }
 template <class T> inline void __stcs(T* p, T v) { *p = v; }
+namespace ichee {
+template <class F> cudaError_t cudaFuncSetAttribute(F*, cudaFuncAttribute, int) { return cudaSuccess; }
+}
 inline unsigned atomicAdd(unsigned* p, unsigned v) { const unsigned o = *p; *p += v; return o; }
 '''
 
@@ -124,9 +127,6 @@ COMMON = r'''
 #include "internal.h"
 #include <algorithm>
 #include <random>
-namespace ichee {
-template <class F> cudaError_t cudaFuncSetAttribute(F*, cudaFuncAttribute, int) { return cudaSuccess; }
-}
 using namespace ichee;
 namespace hm = ichee::host;
 static std::mt19937_64 rng(1);
@@ -346,8 +346,9 @@ int main() { return check<10>() + check<11>() + check<12>() + check<13>() + chec
 BAR = 'asm volatile("bar.sync %0, %1;" ::"r"(first + group), "n"(T / groups) : "memory");'
 
 
-@pytest.mark.parametrize("name,main", [("kernels_enc", ENC), ("kernels_match", MATCH)], ids=["encryption", "matching"])
-def test_results_do_not_depend_on_the_order_of_the_warps(name, main, tmp_path):
+def run_on_host(name, main, tmp_path):
+    """Compile `main` for the CPU, with the shim and the source of csrc/<name>.cu (launches cut out) as
+    <name>_host.h, and run it; a failure shows what it printed."""
     cxx, cc = shutil.which("g++"), nvcc()
     if cxx is None or cc is None:
         pytest.skip("g++ or the CUDA headers not found")
@@ -371,3 +372,8 @@ def test_results_do_not_depend_on_the_order_of_the_warps(name, main, tmp_path):
     assert r.returncode == 0, r.stderr[-4000:]
     r = subprocess.run([str(exe)], capture_output=True, text=True, timeout=600)
     assert r.returncode == 0, r.stdout + r.stderr
+
+
+@pytest.mark.parametrize("name,main", [("kernels_enc", ENC), ("kernels_match", MATCH)], ids=["encryption", "matching"])
+def test_results_do_not_depend_on_the_order_of_the_warps(name, main, tmp_path):
+    run_on_host(name, main, tmp_path)
