@@ -57,9 +57,9 @@ __device__ __forceinline__ void tensor_terms(u64* acc, const u64 (&r)[2][E], int
 // transforms' outputs below 4q as the Montgomery products take them, the accumulators in [0, 2q).
 // Moduli below 2^50 (NOFOLD) need no reduction inside a transform at all.
 // Whole matching calls, 4096 pairs at N = 2^13 with primes 60/40/60: 2.59 ms with a conditional
-// subtraction per butterfly, exact quotients and canonical values, 2.31 lazily reduced, 2.23 with the
-// exchange barriers of ntt.cuh, 2.13 with both polynomials at once; 1600 pairs at N = 2^12 0.74, 0.55,
-// 0.52 and 0.50. What bounds it: the multiply pipe, three quarters busy; the rest of the time goes
+// subtraction per butterfly, exact quotients and canonical values, 2.31 lazily reduced, 2.27 with the
+// exchange barriers of ntt.cuh, 2.24 with the short relinearisation below, 2.15 with both polynomials at
+// once; 1600 pairs at N = 2^12 0.74 ms at first, 0.52 with the short relinearisation, 0.50 now. What bounds it: the multiply pipe, three quarters busy; the rest of the time goes
 // to exchanges and to the tensor terms' accumulators (in L2).
 template <int LOGN, int E, int CAP>
 __device__ __forceinline__ void sqdiff_accumulate(const SqDiffArgs& a, u64* buf)
@@ -116,9 +116,9 @@ __device__ __forceinline__ void sqdiff_accumulate(const SqDiffArgs& a, u64* buf)
                     const int x = elem_offset<LOGN, 0, E>(e);
                     r[e] = __ldcs(pa + x) + q - __ldcs(pb + x);
                 }
-                // d0 is transformed in its parking buffer and d1 in the other one: d1's transform then
-                // starts after d0's block-wide exchanges, which every thread reaches only after its
-                // reads of the previous pixel, so it needs no barrier of its own. Every thread parks
+                // d0 is transformed in its parking buffer and d1 in the other one: the barrier before d0's
+                // transform is past every thread's reads of the previous pixel from either buffer, so
+                // d1's transform needs none of its own. Every thread parks
                 // and reads back only the slots of its own last-pass registers -- the slots it loaded
                 // in the transform's last exchange -- so no barrier follows the transform.
                 if (p == 0) __syncthreads();
@@ -322,8 +322,8 @@ cudaError_t launch_reduce_rows(const RnsArgs& rns, int rows, int limbs, const u6
 // last pass (inverse), and its last exchange loads the slots of the other end, so a block
 // barrier is needed only between two transforms of the same direction: after a forward, an
 // inverse overwrites only slots its thread loaded last, and after an inverse a forward does.
-// 4096 pairs at N = 2^13 and three limbs take 11.1 ms (11.9 with a subtraction per butterfly, exact
-// quotients and canonical accumulators), 768 at N = 2^14 and five limbs 13.2 ms.
+// 4096 pairs at N = 2^13 and three limbs take 11.0 ms (11.9 with a subtraction per butterfly, exact
+// quotients and canonical accumulators), 768 at N = 2^14 and five limbs 13.3 ms.
 // Every intermediate word is produced and consumed by the same thread (the transforms move
 // data between threads only through their own shared buffer), so the block's scratch
 // ([3 limbs + 2][N] words: t0^, t1^, t2 per limb, then the two P accumulators) is stored

@@ -138,7 +138,7 @@ __host__ __device__ constexpr unsigned full_exchanges_in_warp(int logn, int E)
 // An exchange that leaves the warp need not be a barrier of the block: only warps whose numbers
 // differ in bits that the exchange moves trade data. Mask of the warp-number bits (thread bits from 5
 // up) that stay on the same index bit in both layouts, at most the three highest. The groups drift
-// apart, so that one computes while another exchanges: matching at N = 2^13 2.31 -> 2.26 ms, at 2^14
+// apart, so that one computes while another exchanges: matching at N = 2^13 2.31 -> 2.27 ms, at 2^14
 // 6.60 -> 6.44 ms.
 __host__ __device__ constexpr int exchange_fixed_bits(int logn, int sa, int sb, int E)
 {
@@ -475,7 +475,7 @@ __device__ __forceinline__ void load_sm_rt(const u64* sm, u64 (&r)[E], int tid, 
 // Forward stages S0 .. S0+LE-1 (lo = LOGN - S0 - LE): registers below CAP q on entry and exit (one
 // code for every pass, so every stage halves its first operands). The runtime passes take the exact
 // quotient: the three-product form spilled more there (312 against 184 bytes; per-pixel squared
-// difference of 768 pairs at N = 2^14 16.9 against 13.8 ms).
+// difference of 768 pairs at N = 2^14 16.9 against 13.3 ms).
 template <int CAP, int E = 16>
 __device__ __forceinline__ void fwd_regs_rt(u64 (&r)[E], int tid, int S0, int lo, const ulonglong2* __restrict__ tw, u64 q)
 {

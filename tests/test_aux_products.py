@@ -128,7 +128,7 @@ def test_reconstruction_modulo_the_limb(logn):
     dict(log_n=11, prime_bits=[60, 30, 44, 45], log2_scale=25),
     dict(log_n=12, prime_bits=[43, 44], log2_scale=30),
     dict(log_n=13, prime_bits=[41, 42, 43], log2_scale=30),
-    dict(log_n=14, prime_bits=[41, 40, 60, 42], log2_scale=30),        # v^ of the third prime made again per limb
+    dict(log_n=14, prime_bits=[41, 40, 60, 42], log2_scale=30),        # the third prime's digits wait in the output
 ], ids=lambda r: "n%d" % (1 << r["log_n"]))
 def test_fresh_against_the_oracle(ring):
     torch = pytest.importorskip("torch")
