@@ -1235,7 +1235,14 @@ static int sqdiff_blocks(const ichee_ctx* c, int limbs, u64 n_ct)
 
 static size_t sqdiff_slice_words(const ichee_ctx* c) { return (size_t)(sqdiff_split(c->logn) ? 2 : 4) * c->n; }
 
-static size_t relin_words(const ichee_ctx* c, int limbs) { return ichee::relin_words(c->logn, limbs); }
+// Words of the relinearisation working set: the tensor [3][limbs][N], the key-switching digits,
+// the accumulators over Q*P and t2 in the coefficient domain (in the room of a ciphertext).
+static size_t relin_words(const ichee_ctx* c, int limbs)
+{
+    const size_t n = (size_t)c->n;
+    return (size_t)3 * limbs * n + (size_t)limbs * (limbs + 1) * n + (size_t)2 * (limbs + 1) * n +
+           (size_t)2 * limbs * n;
+}
 
 // tensor (= or +=) sum over the pixel pairs of (a - b) (x) (a - b), in the NTT domain (every term
 // carries the Montgomery factor 2^-64); partial: n_blocks x 4N words of scratch.

@@ -175,11 +175,7 @@ cudaError_t launch_sqdiff_image(const SqImgArgs& a, int grid, cudaStream_t st);
 // Relinearisation and rescale of a degree-2 ciphertext tensor[3][limbs][N] in the transform domain
 // (residues below each prime, with the Montgomery factor 2^{-64}) into a.out (one ciphertext of
 // limbs - 1 limbs); a's keys and constants, not its inputs. Working memory: t2 [limbs][N], digits
-// [limbs][limbs + 1][N], acc [2][limbs + 1][N]; relin_words counts these and the tensor.
-inline size_t relin_words(int logn, int limbs)
-{
-    return (size_t)(3 * limbs + limbs + limbs * (limbs + 1) + 2 * (limbs + 1)) << logn;
-}
+// [limbs][limbs + 1][N], acc [2][limbs + 1][N].
 cudaError_t launch_relin_rescale(const SqImgArgs& a, const u64* tensor, u64* t2, u64* digits, u64* acc, cudaStream_t st);
 
 }  // namespace ichee
